@@ -121,7 +121,12 @@ typedef struct {
                               thinning one table (the one `prefilter` names; the larger,
                               S on a tie, when both are named).  Auto = 2 unless the
                               columns are read in place from host memory or more than
-                              18 partition bits are needed                              */
+                              18 partition bits are needed.  With this and the other
+                              partition knobs (prefilter, radix_bits, radix_bits1,
+                              filter_bits, heavy, table_rows) left automatic, a hash
+                              join whose smaller table has at most 2^22 rows is not
+                              partitioned at all: one hash table of that table in
+                              global memory, probed by the other                        */
     int32_t table_rows;    /* R rows per shared-memory table of the hash and sort-merge
                               joins (the "bucket" a work item holds): 0 = the key type's
                               full table (4096 rows for int32 keys, 2048 for int64),
@@ -164,8 +169,10 @@ typedef struct {
                                    cross regions, or |R| * |S| for the nested loop;
                                    always >= result                                 */
     uint64_t hash_path;         /* partition path taken by the hash / sort-merge join:
-                                   1 two radix passes, 2 regions (see jn_tuning)     */
-    uint64_t table_rows;        /* R rows per shared-memory table the join used     */
+                                   1 two radix passes, 2 regions, 3 none: one table
+                                   in global memory (see jn_tuning)                  */
+    uint64_t table_rows;        /* R rows per shared-memory table the join used
+                                   (0 when not partitioned)                          */
     uint64_t reserved[1];
 } jn_run_info;
 
@@ -223,7 +230,8 @@ jn_status jn_aggregate(jn_ctx* ctx, int32_t algo, const jn_table* R, const jn_ta
  * *n_out (host) receives the number of pairs written. */
 
 /* Star join: the multi-table join Sec. 6 leaves to future work, as two of
- * this library's hash joins (a left-deep plan).  R carries two join columns,
+ * this library's hash joins (a left-deep plan), or in one pass over R when
+ * the hash tables of S1 and S2 fit the GPU's L2.  R carries two join columns,
  * key (fk1) and key2 (fk2); every row m of R, n1 of S1 and n2 of S2 with
  * R.key[m] == S1.key[n1] and R.key2[m] == S2.key[n2] gives one triple.
  *   - All key columns share one key type.  R's key2 and payload must be

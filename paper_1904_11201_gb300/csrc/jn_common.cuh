@@ -44,6 +44,8 @@ enum KernelId {
     K_REGION2,
     K_THETA_GATHER,
     K_STAR,
+    K_DIRECT_BUILD,
+    K_DIRECT_PROBE,
     K_COUNT_IDS
 };
 
@@ -119,9 +121,12 @@ struct Scratch {
     std::vector<void*> ptrs;
     uint64_t held = 0;
     explicit Scratch(jn_ctx* ctx) : c(ctx) {}
-    ~Scratch() {
+    ~Scratch() { release(); }
+    void release() {  // frees what is held now
         for (void* p : ptrs) dfree(c, p);
+        ptrs.clear();
         c->scratch_bytes -= held;
+        held = 0;
     }
     template <typename T>
     jn_status get(T** p, size_t count) {

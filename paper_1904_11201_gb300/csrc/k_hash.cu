@@ -827,6 +827,11 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
         }
         return JN_OK;
     }
+    if (!sort_merge) {
+        bool taken = false;
+        const jn_status st = run_direct<K>(c, R, S, mode, plan, res, &taken);
+        if (st != JN_OK || taken) return st;
+    }
     const jn_tuning& tu = c->tune;
     // ---- parameters ----
     // R rows per shared-memory table: the full table or half of it (a smaller
