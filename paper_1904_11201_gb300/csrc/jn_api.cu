@@ -244,60 +244,91 @@ template <typename K>
 static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair** out, uint64_t capacity,
                              uint64_t* n_out, uint64_t* first, uint64_t* pairs, bool count_only) {
     Scratch s(c);
-    std::vector<int> eq, bd;
-    for (int i = 0; i < count; i++) (joins[i].band < 0 ? eq : bd).push_back(i);
-    std::vector<Cols<K>> ER(eq.size()), ES(eq.size()), BR(bd.size()), BS(bd.size());
-    std::vector<int> bops(bd.size());
-    std::vector<int64_t> bbands(bd.size());
+    // the batch's parts: equi-joins with a table small enough to stay in L2,
+    // the other equi-joins, band joins; each part runs as one
+    std::vector<int> part[3];
+    for (int i = 0; i < count; i++)
+        part[joins[i].band >= 0 ? 2 : batch_direct_takes(c, joins[i].R.n, joins[i].S.n) ? 0 : 1].push_back(i);
+    std::vector<Cols<K>> cr[3], cs[3];
+    std::vector<int> bops;
+    std::vector<int64_t> bbands;
     HostCopies hc(c);
-    for (size_t j = 0; j < eq.size(); j++) {
-        JN_TRY(stage<K>(c, s, hc, &joins[eq[j]].R, false, &ER[j]));
-        JN_TRY(stage<K>(c, s, hc, &joins[eq[j]].S, false, &ES[j]));
-    }
-    for (size_t j = 0; j < bd.size(); j++) {
-        JN_TRY(stage<K>(c, s, hc, &joins[bd[j]].R, true, &BR[j]));
-        JN_TRY(stage<K>(c, s, hc, &joins[bd[j]].S, true, &BS[j]));
-        bops[j] = joins[bd[j]].op;
-        bbands[j] = joins[bd[j]].band;
+    for (int k = 0; k < 3; k++) {
+        cr[k].resize(part[k].size());
+        cs[k].resize(part[k].size());
+        for (size_t j = 0; j < part[k].size(); j++) {
+            const jn_join& x = joins[part[k][j]];
+            JN_TRY(stage<K>(c, s, hc, &x.R, k == 2, &cr[k][j]));
+            JN_TRY(stage<K>(c, s, hc, &x.S, k == 2, &cs[k][j]));
+            if (k == 2) {
+                bops.push_back(x.op);
+                bbands.push_back(x.band);
+            }
+        }
     }
     JN_TRY(hc.start());
     JN_TRY(wait_copies(c, true));
     // every join is counted before the single output allocation
-    std::unique_ptr<BatchRun> he, be;
-    if (!eq.empty()) JN_TRY(batch_hash_prepare<K>(c, (int)eq.size(), ER.data(), ES.data(), &he));
-    if (!bd.empty())
-        JN_TRY(batch_band_prepare<K>(c, (int)bd.size(), BR.data(), BS.data(), bops.data(), bbands.data(), &be));
-    const uint64_t te = he ? he->total : 0, tb = be ? be->total : 0;
+    std::unique_ptr<BatchRun> run[3];
+    if (!part[0].empty()) {
+        const jn_status st =
+            batch_direct_prepare<K>(c, (int)part[0].size(), cr[0].data(), cs[0].data(), count_only, &run[0]);
+        if (st == JN_ERR_OOM) {
+            // a device too full for the tables and the pairs' room: all of them partitioned
+            c->err.clear();
+            for (size_t j = 0; j < part[0].size(); j++) {
+                part[1].push_back(part[0][j]);
+                cr[1].push_back(cr[0][j]);
+                cs[1].push_back(cs[0][j]);
+            }
+            part[0].clear();
+        } else if (st != JN_OK) {
+            return st;
+        }
+    }
+    if (!part[1].empty())
+        JN_TRY(batch_hash_prepare<K>(c, (int)part[1].size(), cr[1].data(), cs[1].data(), &run[1]));
+    if (!part[2].empty())
+        JN_TRY(batch_band_prepare<K>(c, (int)part[2].size(), cr[2].data(), cs[2].data(), bops.data(), bbands.data(),
+                                     &run[2]));
+    uint64_t total = 0;
+    for (int k = 0; k < 3; k++) total += run[k] ? run[k]->total : 0;
+    auto publish = [&] {
+        uint64_t at = 0;
+        for (int k = 0; k < 3; k++) {
+            for (size_t j = 0; j < part[k].size(); j++) {
+                first[part[k][j]] = at + run[k]->offsets[j];
+                pairs[part[k][j]] = run[k]->offsets[j + 1] - run[k]->offsets[j];
+            }
+            at += run[k] ? run[k]->total : 0;
+        }
+    };
     if (count_only) {
-        for (size_t j = 0; j < eq.size(); j++) pairs[eq[j]] = he->offsets[j + 1] - he->offsets[j];
-        for (size_t j = 0; j < bd.size(); j++) pairs[bd[j]] = be->offsets[j + 1] - be->offsets[j];
-        *n_out = te + tb;
-        c->info.result = te + tb;
+        publish();
+        *n_out = total;
+        c->info.result = total;
         return JN_OK;
     }
     OutPlan plan;
     plan.user_out = out;
     plan.capacity = capacity;
     plan.n_out = n_out;
-    JN_TRY(out_prepare(c, s, te + tb, plan));
+    JN_TRY(out_prepare(c, s, total, plan));
     if (plan.host_copy && !is_device_pointer(*out))
         return fail(c, JN_ERR_INVALID, "batch outputs must be device memory");
-    if (he) JN_TRY(he->emit(c, plan.dev));
-    if (be) JN_TRY(be->emit(c, plan.dev + te));
-    for (size_t j = 0; j < eq.size(); j++) {
-        first[eq[j]] = he->offsets[j];
-        pairs[eq[j]] = he->offsets[j + 1] - he->offsets[j];
+    uint64_t at = 0;
+    for (int k = 0; k < 3; k++) {
+        if (!run[k]) continue;
+        JN_TRY(run[k]->emit(c, plan.dev + at));
+        at += run[k]->total;
     }
-    for (size_t j = 0; j < bd.size(); j++) {
-        first[bd[j]] = te + be->offsets[j];
-        pairs[bd[j]] = be->offsets[j + 1] - be->offsets[j];
-    }
-    JN_TRY(out_finish(c, te + tb, plan));
+    publish();
+    JN_TRY(out_finish(c, total, plan));
     uint64_t dummy;
     uint64_t* d_small;
     JN_TRY(s.get(&d_small, 1));
     JN_TRY(read_back(c, d_small, &dummy, 0));  // reports a device wait that ran out
-    c->info.result = te + tb;
+    c->info.result = total;
     return JN_OK;
 }
 

@@ -174,14 +174,15 @@ __device__ __forceinline__ uint32_t dj_claim(const DirectTab<K, MODE>& t, K k) {
 // Inserts the build rows.  Emit: where[i] = (slot, rank among the key's
 // rows), and the rank-0 row leaves its payload in the slot, which is final
 // when no key has several rows.  use_g: the build side is S.
+// The block takes rows [b0, b0 + DJ_T), then the next DJ_T `stride` further, of
+// [0, n); so do the other loops over rows here.
 template <typename K, int MODE>
-__global__ void __launch_bounds__(DJ_T)
-k_direct_insert(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int use_g,
-                uint2* __restrict__ where, DirectSmall* __restrict__ small) {
+__device__ __forceinline__ void dj_insert_rows(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t b0,
+                                               int64_t n, int64_t stride, const DirectTab<K, MODE>& t, int use_g,
+                                               uint2* __restrict__ where, DirectLine* __restrict__ line) {
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * DJ_T;
     bool dup = false;
-    for (int64_t b = (int64_t)blockIdx.x * DJ_T + threadIdx.x - lane; b < n; b += stride) {
+    for (int64_t b = b0 + threadIdx.x - lane; b < n; b += stride) {
         const int64_t i = b + lane;
         const bool in = i < n;
         const unsigned act = __ballot_sync(0xffffffffu, in);
@@ -212,19 +213,26 @@ k_direct_insert(const K* __restrict__ key, const int32_t* __restrict__ pay, int6
                 dup = true;
         }
     }
-    if (MODE == MODE_EMIT && dup) small->lines[0].dup = 1;
+    if (MODE == MODE_EMIT && dup) line->dup = 1;
+}
+
+template <typename K, int MODE>
+__global__ void __launch_bounds__(DJ_T)
+k_direct_insert(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int use_g,
+                uint2* __restrict__ where, DirectSmall* __restrict__ small) {
+    dj_insert_rows<K, MODE>(key, pay, (int64_t)blockIdx.x * DJ_T, n, (int64_t)gridDim.x * DJ_T, t, use_g, where,
+                            small->lines);
 }
 
 // Some key has several rows (nothing to do otherwise): the rank-0 row of a
 // key reserves its run and leaves the start in the slot.
 template <typename K>
-__global__ void __launch_bounds__(DJ_T)
-k_direct_runs(int64_t n, DirectTab<K, MODE_EMIT> t, const uint2* __restrict__ where, DirectSmall* __restrict__ small) {
-    if (!small->lines[0].dup) return;
+__device__ __forceinline__ void dj_runs_rows(int64_t b0, int64_t n, int64_t stride, const DirectTab<K, MODE_EMIT>& t,
+                                             const uint2* __restrict__ where, DirectLine* __restrict__ line) {
+    if (!line->dup) return;
     constexpr bool HEAD = DirectSlot<K, MODE_EMIT>::COUNTS_ASIDE;  // runs begin with their length
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * DJ_T;
-    for (int64_t b = (int64_t)blockIdx.x * DJ_T + threadIdx.x - lane; b < n; b += stride) {
+    for (int64_t b = b0 + threadIdx.x - lane; b < n; b += stride) {
         const int64_t i = b + lane;
         uint2 w = make_uint2(0, 1);
         if (i < n) w = where[i];
@@ -234,7 +242,7 @@ k_direct_runs(int64_t n, DirectTab<K, MODE_EMIT> t, const uint2* __restrict__ wh
         const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
         if (tot == 0) continue;
         uint32_t at = 0;
-        if (lane == 0) at = (uint32_t)atomicAdd(&small->lines[0].cursor, (unsigned long long)tot);
+        if (lane == 0) at = (uint32_t)atomicAdd(&line->cursor, (unsigned long long)tot);
         at = __shfl_sync(0xffffffffu, at, 0) + incl - c;
         if (c) {
             *t.value_at(w.x) = at;
@@ -243,18 +251,30 @@ k_direct_runs(int64_t n, DirectTab<K, MODE_EMIT> t, const uint2* __restrict__ wh
     }
 }
 
+template <typename K>
+__global__ void __launch_bounds__(DJ_T)
+k_direct_runs(int64_t n, DirectTab<K, MODE_EMIT> t, const uint2* __restrict__ where, DirectSmall* __restrict__ small) {
+    dj_runs_rows<K>((int64_t)blockIdx.x * DJ_T, n, (int64_t)gridDim.x * DJ_T, t, where, small->lines);
+}
+
 // ... and every row writes its payload into its key's run.
+template <typename K>
+__device__ __forceinline__ void dj_place_rows(const int32_t* __restrict__ pay, int64_t b0, int64_t n, int64_t stride,
+                                              const DirectTab<K, MODE_EMIT>& t, const uint2* __restrict__ where,
+                                              const DirectLine* __restrict__ line) {
+    if (!line->dup) return;
+    constexpr bool HEAD = DirectSlot<K, MODE_EMIT>::COUNTS_ASIDE;
+    for (int64_t i = b0 + threadIdx.x; i < n; i += stride) {
+        const uint2 w = where[i];
+        if (HEAD || *t.rows_at(w.x) > 1) t.runs[*t.value_at(w.x) + HEAD + w.y] = pay ? pay[i] : (int32_t)i;
+    }
+}
+
 template <typename K>
 __global__ void __launch_bounds__(DJ_T)
 k_direct_place(const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE_EMIT> t, const uint2* __restrict__ where,
                const DirectSmall* __restrict__ small) {
-    if (!small->lines[0].dup) return;
-    constexpr bool HEAD = DirectSlot<K, MODE_EMIT>::COUNTS_ASIDE;
-    const int64_t stride = (int64_t)gridDim.x * DJ_T;
-    for (int64_t i = (int64_t)blockIdx.x * DJ_T + threadIdx.x; i < n; i += stride) {
-        const uint2 w = where[i];
-        if (HEAD || *t.rows_at(w.x) > 1) t.runs[*t.value_at(w.x) + HEAD + w.y] = pay ? pay[i] : (int32_t)i;
-    }
+    dj_place_rows<K>(pay, (int64_t)blockIdx.x * DJ_T, n, (int64_t)gridDim.x * DJ_T, t, where, small->lines);
 }
 
 // Looks U keys up, a step of all of them in flight together.  m[u]: rows of
@@ -379,28 +399,21 @@ struct WarpOut {
     }
 };
 
-// Probes the table with n rows.  Emit writes the pairs in WarpOut's manner to
-// `segs` segments of `cap` pairs each, block b to segment b mod segs (the
-// segments' totals count pairs past `cap` too).  swap: the build side is S.
+// Probes the table with the block's rows (of DJ_U * DJ_T at a time).  Emit:
+// pairs go out through `wo`, which keeps what it has not written yet.
+// Count and aggregate add to acc and csum.  swap: the build side is S.
 //
 // Bound by the latency of the bucket reads, so what matters is how many are
 // in flight: small blocks at full occupancy, the next rows' keys and payloads
 // loading while these are looked up, payloads read whether or not their row
 // matches.
 template <typename K, int MODE>
-__global__ void __launch_bounds__(DJ_T, JN_DJ_MINB)
-k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int swap,
-               DirectSmall* __restrict__ small, jn_pair* __restrict__ out, uint32_t segs, unsigned long long cap) {
-    constexpr int U = DJ_U, TILE = DJ_T * U;
-    using Out = WarpOut<2>;
-    __shared__ int2 s_buf[MODE == MODE_EMIT ? DJ_T / 32 : 1][MODE == MODE_EMIT ? Out::ROOM : 1];
+__device__ __forceinline__ void dj_probe_rows(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t b0,
+                                              int64_t n, int64_t stride, const DirectTab<K, MODE>& t, int swap,
+                                              WarpOut<2>& wo, unsigned long long& acc, unsigned long long& csum) {
+    constexpr int U = DJ_U;
     const int lane = threadIdx.x & 31;
-    const uint32_t seg = blockIdx.x % segs;
-    out += seg * cap;
-    Out wo{MODE == MODE_EMIT ? s_buf[threadIdx.x >> 5] : nullptr, &small->lines[seg].total,
-           reinterpret_cast<int2*>(out), cap, 0};
     const bool dup = MODE == MODE_EMIT && *t.dup != 0;
-    unsigned long long acc = 0, csum = 0;
     K kn[U];
     int32_t pn[U];
     auto load = [&](int64_t t0) {
@@ -411,9 +424,9 @@ k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64
             if (MODE != MODE_COUNT) pn[u] = pay && i < n ? __ldcs(pay + i) : (int32_t)i;
         }
     };
-    int64_t t0 = (int64_t)blockIdx.x * TILE;
+    int64_t t0 = b0;
     load(t0);
-    for (; t0 < n; t0 += (int64_t)gridDim.x * TILE) {
+    for (; t0 < n; t0 += stride) {
         K k[U];
         int32_t pp[U];
         bool valid[U];
@@ -425,7 +438,7 @@ k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64
             pp[u] = pn[u];
             valid[u] = t0 + u * DJ_T + threadIdx.x < n;
         }
-        load(t0 + (int64_t)gridDim.x * TILE);
+        load(t0 + stride);
         dj_lookup<K, MODE, U>(t, dup, k, valid, m, v, fs);
         if (MODE == MODE_EMIT) {
 #pragma unroll
@@ -443,7 +456,7 @@ k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64
                 const unsigned long long incl = warp_incl_scan((unsigned long long)m[u]);
                 unsigned long long at;
                 if (!wo.reserve(__shfl_sync(0xffffffffu, incl, 31), &at)) continue;
-                jn_pair* o = out + at + (incl - m[u]);
+                jn_pair* o = reinterpret_cast<jn_pair*>(wo.out) + at + (incl - m[u]);
                 if (m[u] <= 4) {
                     for (uint32_t e = 0; e < m[u]; e++) {
                         const int32_t bp = dj_single<K>(dup, m[u]) ? (int32_t)v[u] : t.runs[v[u] + e];
@@ -472,6 +485,24 @@ k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64
             }
         }
     }
+}
+
+// The single join's probe.  Emit: `segs` segments of `cap` pairs each at out,
+// block b to segment b mod segs (the segments' totals count pairs past `cap`
+// too).
+template <typename K, int MODE>
+__global__ void __launch_bounds__(DJ_T, JN_DJ_MINB)
+k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int swap,
+               DirectSmall* __restrict__ small, jn_pair* __restrict__ out, uint32_t segs, unsigned long long cap) {
+    constexpr int TILE = DJ_T * DJ_U;
+    using Out = WarpOut<2>;
+    __shared__ int2 s_buf[MODE == MODE_EMIT ? DJ_T / 32 : 1][MODE == MODE_EMIT ? Out::ROOM : 1];
+    const uint32_t seg = blockIdx.x % segs;
+    out += seg * cap;
+    Out wo{MODE == MODE_EMIT ? s_buf[threadIdx.x >> 5] : nullptr, &small->lines[seg].total,
+           reinterpret_cast<int2*>(out), cap, 0};
+    unsigned long long acc = 0, csum = 0;
+    dj_probe_rows<K, MODE>(key, pay, (int64_t)blockIdx.x * TILE, n, (int64_t)gridDim.x * TILE, t, swap, wo, acc, csum);
     if (MODE == MODE_EMIT) {
         wo.flush();
     } else {
