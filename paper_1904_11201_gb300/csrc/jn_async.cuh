@@ -74,6 +74,11 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t
         : "memory");
 }
 
+// Starts bringing `bytes` (multiple of 16) at `src` (16-byte aligned) to L2.
+__device__ __forceinline__ void l2_prefetch(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // Rows [beg, beg + cnt) of an array of E-byte elements, widened to 16-byte
 // boundaries: the copy starts at row a0 = beg rounded down and spans `bytes`.
 // `rows_ok` is how many rows of the array may be read (allocation size);

@@ -628,18 +628,30 @@ struct DirectResult {
     uint64_t total = 0, chk = 0, first = 0;
     bool fits = true;  // every segment's results fit its room
 };
-inline jn_status direct_result(jn_ctx* c, const DirectSmall* small, uint32_t segs, uint64_t cap, DirectResult* r) {
+// Queues the counters' copy to the host; after the stream is synchronised,
+// direct_parse reads them.
+constexpr int DJ_HWORD = 16;  // where they land in the context's pinned words
+inline jn_status direct_fetch(jn_ctx* c, const DirectSmall* small, uint32_t segs) {
     constexpr int W = 4;  // words of a line that matter here
-    JN_CUDA(c, cudaMemcpy2DAsync(c->h_small, W * 8, small, sizeof(DirectLine), W * 8, segs, cudaMemcpyDeviceToHost,
-                                 c->stream));
-    JN_CUDA(c, cudaStreamSynchronize(c->stream));
+    static_assert(DJ_HWORD + W * DJ_SEGS < 63, "the last pinned word is read_back's error word");
+    JN_CUDA(c, cudaMemcpy2DAsync(c->h_small + DJ_HWORD, W * 8, small, sizeof(DirectLine), W * 8, segs,
+                                 cudaMemcpyDeviceToHost, c->stream));
+    return JN_OK;
+}
+inline void direct_parse(const jn_ctx* c, uint32_t segs, uint64_t cap, DirectResult* r) {
+    const uint64_t* h = c->h_small + DJ_HWORD;
     for (uint32_t i = 0; i < segs; i++) {
-        r->counts.n[i] = c->h_small[W * i];
+        r->counts.n[i] = h[4 * i];
         r->total += r->counts.n[i];
         r->fits &= r->counts.n[i] <= cap;
     }
-    r->chk = c->h_small[1];
-    r->first = c->h_small[2];
+    r->chk = h[1];
+    r->first = h[2];
+}
+inline jn_status direct_result(jn_ctx* c, const DirectSmall* small, uint32_t segs, uint64_t cap, DirectResult* r) {
+    JN_TRY(direct_fetch(c, small, segs));
+    JN_CUDA(c, cudaStreamSynchronize(c->stream));
+    direct_parse(c, segs, cap, r);
     return JN_OK;
 }
 

@@ -11,17 +11,19 @@
 //   3. partition pass 2 (b2 more bits), exact offsets from a histogram of
 //      the pass-1 output.  Partition p = top (b1 + b2) hash bits; the pair of
 //      passes plays the role of the shuffle on join_key / alpha.
-//   4. work items (partition, R chunk, S chunk); count pass builds a
-//      shared-memory hash table on the R chunk and probes with the S chunk;
-//      exclusive scan of the per-item counts gives exact output offsets and
-//      the total (one 8-byte read-back).
-//   5. one exact allocation, then the emit pass repeats build and probe and
-//      writes (R.payload, S.payload) pairs at the scanned offsets.
+//   4. work items (partition, R chunk); the join kernel builds a shared-memory
+//      hash table on the R chunk, probes it with the partition's S rows and
+//      keeps the pairs it finds in scratch (jn_partjoin.cuh).
+//   5. one exact allocation (the total is one 8-byte read-back) and one copy.
+//      Inputs with many frequent keys, and the sort-merge join, count per item
+//      in step 4, scan the counts to output offsets, and join a second time to
+//      write the pairs there.
 #include <vector>
 
 #include "jn_algos.h"
 #include "jn_heavy.cuh"
 #include "jn_partition.cuh"
+#include "jn_partjoin.cuh"
 #include "jn_region.cuh"
 #include "jn_sortjoin.cuh"
 
@@ -160,6 +162,8 @@ __device__ __forceinline__ uint32_t oa_slot(uint32_t h, int bits, int ts) {
     return (uint32_t)(((uint64_t)x * (uint64_t)ts) >> 32);
 }
 
+// The join kernel of inputs with many frequent keys (MERGE) and of batches;
+// the others take k_part_join.
 // MODE_COUNT: item_val[it] = matches of the item.
 // MODE_AGG:   as COUNT, and chk += sum over matches of f(r) * g(s).
 // MODE_EMIT:  writes the item's pairs at out[item_off[it] ...].
@@ -572,13 +576,12 @@ static size_t hash_smem(int mode, int cap = cap_of<K>()) {
     return cap == C ? JoinSmem<K, MODE_COUNT>::BYTES : JoinSmem<K, MODE_COUNT, H>::BYTES;
 }
 
-// The join kernel for a table of `cap` R rows (the full table or half of it),
-// with or without the skewed-input build.
+// The skewed-input join kernel for a table of `cap` R rows (the full table or
+// half of it).
 template <typename K, int MODE>
-static auto hash_join_kernel(bool merge, int cap) {
+static auto hash_join_kernel(int cap) {
     constexpr int C = cap_of<K>(), H = C / 2;
-    if (cap == C) return merge ? k_hash_join<K, MODE, true, C> : k_hash_join<K, MODE, false, C>;
-    return merge ? k_hash_join<K, MODE, true, H> : k_hash_join<K, MODE, false, H>;
+    return cap == C ? k_hash_join<K, MODE, true, C> : k_hash_join<K, MODE, true, H>;
 }
 
 static int persistent_grid(jn_ctx* c, const void* fn, int threads, size_t smem) {
@@ -838,7 +841,7 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     // table doubles the partitions for the same rows per partition); a size
     // outside the key type's two is taken as the nearer one, so one context
     // serves both key types
-    const int cap = tu.table_rows == 0 || tu.table_rows >= cap_of<K>() ? cap_of<K>() : cap_of<K>() / 2;
+    int cap = tu.table_rows == 0 || tu.table_rows >= cap_of<K>() ? cap_of<K>() : cap_of<K>() / 2;
     bool heavy = tu.heavy >= 1 || (tu.heavy == -1 && nr + ns >= (1u << 20));
     const int64_t heavy_rows = tu.heavy >= 2 ? tu.heavy : cap_of<K>() / 4;  // rows that make a key heavy
     // which tables the pre-filter thins: bit 0 S (by R's keys), bit 1 R (by S's keys)
@@ -1010,6 +1013,14 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
         JN_TRY(region ? region_all(d1) : pass_all(d1));
     }
     // ---- 4. work items and the count pass ----
+    const int table_rows = cap;
+    if (!sort_merge && !heavy && tu.table_rows == 0) {
+        // no larger a table than the partitions need (an eighth more than their
+        // rows and 64: six standard deviations of a random 1024), so that three
+        // blocks share an SM; a larger partition is joined in several chunks
+        const uint64_t per = nr / (uint64_t)P;
+        cap = (int)min((uint64_t)cap, max((uint64_t)256, (per + per / 8 + 64 + 127) & ~(uint64_t)127));
+    }
     uint64_t *items, *iprefix;
     JN_TRY(s.get(&items, P));
     JN_TRY(s.get(&iprefix, P + 1));
@@ -1033,20 +1044,60 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     info.radix_bits1 = b1;
     info.filter_bits = fside ? fb : 0;
     info.hash_path = region ? 2 : 1;
-    info.table_rows = (uint64_t)cap;
+    info.table_rows = (uint64_t)table_rows;
     info.heavy_keys = 0;
     // the join kernel stages rows with 16-byte bulk copies from these arrays
     if ((((uintptr_t)PR.rows) | ((uintptr_t)PS.rows)) & 15)
         return fail(c, JN_ERR_CUDA, "partition scratch is not 16-byte aligned");
     Item* idesc;
-    unsigned long long *ival, *chk;
-    uint64_t* ioff;
+    unsigned long long *ival = nullptr, *chk;
+    uint64_t* ioff = nullptr;
     JN_TRY(s.get(&idesc, nitems + 1));
-    JN_TRY(s.get(&ival, nitems + 1));
     RW* rsorted = nullptr;  // sort-merge: the R chunks sorted by key
-    JN_TRY(s.get(&ioff, nitems + 1));
-    JN_TRY(s.get(&chk, 1));
-    JN_TRY(zero(c, chk, 8));
+    // once: the hash join of an input without many frequent keys finds its
+    // pairs and keeps them in one pass (jn_partjoin.cuh); the others count per
+    // item, scan, and join again to write
+    const bool once = !sort_merge && !skewed;
+    const int jcap = cap == cap_of<K>() / 2 ? cap : cap_of<K>();  // k_hash_join comes in two sizes
+    DirectSmall* small = nullptr;
+    jn_pair* staged = nullptr;
+    uint32_t segs = 1;
+    uint64_t room = 0;  // pairs per segment
+    Scratch ss(c);
+    if (once) {
+        JN_TRY(s.get(&small, 1));
+        JN_TRY(zero(c, small, sizeof(DirectSmall)));
+        chk = &small->lines[0].chk;
+        if (mode == MODE_EMIT && nitems && !c->mem_limit && !c->admit) {
+            // random keys on both sides match a surviving row 1.6 times; not
+            // under a limit that counts scratch
+            const uint64_t rows = max(h[0], h[1]);
+            segs = rows >= (1u << 23) ? DJ_SEGS : 1;
+            room = (rows + rows / 4 * 3) / segs + 4096;
+            if (ss.get(&staged, segs * room) != JN_OK) {
+                c->err.clear();
+                segs = 1;
+                room = 0;
+            }
+        }
+    } else {
+        JN_TRY(s.get(&ival, nitems + 1));
+        JN_TRY(s.get(&ioff, nitems + 1));
+        JN_TRY(s.get(&chk, 1));
+        JN_TRY(zero(c, chk, 8));
+    }
+    auto join_once = [&](int m, jn_pair* to, uint32_t parts, uint64_t most) -> jn_status {
+        auto kj = m == MODE_EMIT ? k_part_join<K, MODE_EMIT>
+                  : m == MODE_AGG ? k_part_join<K, MODE_AGG>
+                                  : k_part_join<K, MODE_COUNT>;
+        const size_t sm = m == MODE_EMIT ? PartJoinSmem<K, MODE_EMIT>::bytes(cap)
+                          : m == MODE_AGG ? PartJoinSmem<K, MODE_AGG>::bytes(cap)
+                                          : PartJoinSmem<K, MODE_COUNT>::bytes(cap);
+        const int g = (int)min((uint64_t)persistent_grid(c, (const void*)kj, PJ_T, sm), nitems);
+        return launch(c, m == MODE_EMIT ? K_HASH_EMIT : K_HASH_COUNT, kj, dim3(g), dim3(PJ_T), sm, (const RW*)PR.rows,
+                      (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P), cap, b, small, to, parts,
+                      (unsigned long long)most, c->d_err);
+    };
     if (nitems) {
         JN_TRY(launch(c, K_ITEMS, k_item_desc, dim3((unsigned)ceil_div(nitems, 256)), dim3(256), 0, PR.view(),
                       PS.view(), (const uint64_t*)iprefix, P, cap, idesc));
@@ -1065,17 +1116,19 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             JN_TRY(launch(c, K_SORT_COUNT, kc, dim3(gj), dim3(SJ_T), smc, (const RW*)rsorted, (const RW*)PS.rows,
                           (const Item*)idesc, (const uint64_t*)(iprefix + P), cap, ival, chk,
                           (const uint64_t*)nullptr, (jn_pair*)nullptr, (uint64_t)0, ~0ull));
+        } else if (once) {
+            JN_TRY(join_once(room ? MODE_EMIT : cm, staged, segs, room));
         } else {
-            const size_t smc = hash_smem<K>(cm, cap);
-            auto kc = cm == MODE_AGG ? hash_join_kernel<K, MODE_AGG>(skewed, cap)
-                                     : hash_join_kernel<K, MODE_COUNT>(skewed, cap);
+            const size_t smc = hash_smem<K>(cm, jcap);
+            auto kc = cm == MODE_AGG ? hash_join_kernel<K, MODE_AGG>(jcap)
+                                     : hash_join_kernel<K, MODE_COUNT>(jcap);
             const int gj = (int)min((uint64_t)persistent_grid(c, (const void*)kc, HJ_T, smc), nitems);
             JN_TRY(launch(c, K_HASH_COUNT, kc, dim3(gj), dim3(HJ_T), smc, (const RW*)PR.rows, (const RW*)PS.rows,
                           (const Item*)idesc, (const uint64_t*)(iprefix + P), b, ival, chk,
                           (const uint64_t*)nullptr, (jn_pair*)nullptr, c->d_err, (uint64_t)0, ~0ull));
         }
     }
-    JN_TRY(scan_u64(c, reinterpret_cast<const uint64_t*>(ival), ioff, (int64_t)nitems));
+    if (!once) JN_TRY(scan_u64(c, reinterpret_cast<const uint64_t*>(ival), ioff, (int64_t)nitems));
     // ---- heavy keys: c_R(h) * c_S(h) pairs each ----
     uint64_t *hp = nullptr, *hpoff = nullptr, *hch = nullptr, *hchp = nullptr;
     if (heavy) {
@@ -1100,11 +1153,21 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
                       d_small + 5, 1));
         JN_CUDA(c, cudaMemcpyAsync(d_small + 6, d_hcount, 4, cudaMemcpyDeviceToDevice, c->stream));
     }
-    JN_TRY(launch(c, K_MISC, k_copy_words, dim3(1), dim3(32), 0, (const uint64_t*)(ioff + nitems),
-                  d_small + 3, 1));
-    JN_TRY(launch(c, K_MISC, k_copy_words, dim3(1), dim3(32), 0, (const uint64_t*)chk, d_small + 4, 1));
+    if (once) {
+        JN_TRY(direct_fetch(c, small, segs));
+    } else {
+        JN_TRY(launch(c, K_MISC, k_copy_words, dim3(1), dim3(32), 0, (const uint64_t*)(ioff + nitems),
+                      d_small + 3, 1));
+        JN_TRY(launch(c, K_MISC, k_copy_words, dim3(1), dim3(32), 0, (const uint64_t*)chk, d_small + 4, 1));
+    }
     uint64_t hc[4];
     JN_TRY(read_back(c, d_small + 3, hc, 4));
+    DirectResult found;
+    if (once) {
+        direct_parse(c, segs, room, &found);
+        hc[0] = found.total;
+        hc[1] = found.chk;
+    }
     const uint64_t normal = hc[0], heavy_pairs = heavy ? hc[2] : 0;
     const uint64_t total = normal + heavy_pairs;
     res->count = total;
@@ -1115,11 +1178,12 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     info.cartesian_bound = h[15] + heavy_pairs;  // the frequent keys' cross products are exact
     if (mode != MODE_EMIT) return JN_OK;
     // ---- 5. exact allocation and the emit pass ----
+    if (!found.fits) ss.release();
     JN_TRY(out_prepare(c, s, total, *plan));
     // A host output is copied back slice by slice (on the copy stream) while
     // the later slices of the work queue emit: slice k's pairs are the
     // contiguous range [ioff[ib[k]], ioff[ib[k + 1]]).
-    const int nsl = (plan->host_copy && normal >= (uint64_t)JN_SLICE_PAIRS && nitems >= 64) ? 4 : 1;
+    const int nsl = (!once && plan->host_copy && normal >= (uint64_t)JN_SLICE_PAIRS && nitems >= 64) ? 4 : 1;
     uint64_t ib[5], ob[5] = {0, 0, 0, 0, 0};
     for (int k = 0; k <= nsl; k++) ib[k] = nitems * (uint64_t)k / (uint64_t)nsl;
     if (nsl > 1) {
@@ -1139,10 +1203,17 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
                                    cudaMemcpyDefault, c->copy_stream));
         return JN_OK;
     };
-    if (normal > 0) {
-        auto ke = hash_join_kernel<K, MODE_EMIT>(skewed, cap);
+    if (once && normal > 0) {
+        if (room && found.fits) {
+            JN_TRY((direct_gather<uint64_t, 1>(c, K_HASH_EMIT, staged, segs, room, found, plan->dev)));
+        } else {
+            JN_TRY(zero(c, &small->lines[0].total, 8));
+            JN_TRY(join_once(MODE_EMIT, plan->dev, 1, normal));
+        }
+    } else if (normal > 0) {
+        auto ke = hash_join_kernel<K, MODE_EMIT>(jcap);
         auto kse = k_sort_join<K, MODE_EMIT>;
-        const size_t sme = sort_merge ? SortJoinSmem<K>::bytes(cap, MODE_EMIT) : hash_smem<K>(MODE_EMIT, cap);
+        const size_t sme = sort_merge ? SortJoinSmem<K>::bytes(cap, MODE_EMIT) : hash_smem<K>(MODE_EMIT, jcap);
         const uint64_t pg = sort_merge ? (uint64_t)persistent_grid(c, (const void*)kse, SJ_T, sme)
                                        : (uint64_t)persistent_grid(c, (const void*)ke, HJ_T, sme);
         for (int k = 0; k < nsl; k++) {
