@@ -79,6 +79,20 @@ template <typename K>
 jn_status batch_band_prepare(jn_ctx* c, int m, const Cols<K>* Rs, const Cols<K>* Ss, const int* ops,
                              const int64_t* bands, std::unique_ptr<BatchRun>* run);
 
+// Band joins without partitioning (k_band.cu), for the joins it takes.  A
+// join that turns out to have too many candidates is `stopped`: it has no
+// pairs here and is left to the partitioned join.  JN_ERR_OOM: nothing ran.
+struct BandDirect : BatchRun {
+    std::vector<char> stopped;
+    uint64_t checksum = 0;    // aggregate
+    uint64_t candidates = 0;  // rows compared
+    uint64_t buckets = 0, tiles = 0;
+};
+bool band_direct_takes(const jn_ctx* c, int64_t nr, int64_t ns);
+template <typename K>
+jn_status band_direct_prepare(jn_ctx* c, int n, const Cols<K>* Rs, const Cols<K>* Ss, const int* ops,
+                              const int64_t* bands, int mode, std::unique_ptr<BandDirect>* run);
+
 // Captures a sequence of launches on the context's private stream and replays
 // it as a CUDA graph on the context's stream (or runs it directly when graphs
 // are off).  The caller's stream may be the legacy default stream, which

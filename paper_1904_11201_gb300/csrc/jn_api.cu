@@ -244,43 +244,48 @@ template <typename K>
 static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair** out, uint64_t capacity,
                              uint64_t* n_out, uint64_t* first, uint64_t* pairs, bool count_only) {
     Scratch s(c);
-    // the batch's parts: equi-joins with a table small enough to stay in L2,
-    // the other equi-joins, band joins; each part runs as one
-    std::vector<int> part[3];
-    for (int i = 0; i < count; i++)
-        part[joins[i].band >= 0 ? 2 : batch_direct_takes(c, joins[i].R.n, joins[i].S.n) ? 0 : 1].push_back(i);
-    std::vector<Cols<K>> cr[3], cs[3];
-    std::vector<int> bops;
-    std::vector<int64_t> bbands;
+    // the batch's parts: equi-joins with a table small enough to stay in L2
+    // and the others, band joins likewise; each part runs as one
+    constexpr int PARTS = 4;
+    std::vector<int> part[PARTS];
+    for (int i = 0; i < count; i++) {
+        const int64_t nr = joins[i].R.n, ns = joins[i].S.n;
+        part[joins[i].band >= 0 ? (band_direct_takes(c, nr, ns) ? 2 : 3) : batch_direct_takes(c, nr, ns) ? 0 : 1]
+            .push_back(i);
+    }
+    std::vector<Cols<K>> cr[PARTS], cs[PARTS];
+    std::vector<int> bops[PARTS];
+    std::vector<int64_t> bbands[PARTS];
     HostCopies hc(c);
-    for (int k = 0; k < 3; k++) {
+    for (int k = 0; k < PARTS; k++) {
         cr[k].resize(part[k].size());
         cs[k].resize(part[k].size());
         for (size_t j = 0; j < part[k].size(); j++) {
             const jn_join& x = joins[part[k][j]];
-            JN_TRY(stage<K>(c, s, hc, &x.R, k == 2, &cr[k][j]));
-            JN_TRY(stage<K>(c, s, hc, &x.S, k == 2, &cs[k][j]));
-            if (k == 2) {
-                bops.push_back(x.op);
-                bbands.push_back(x.band);
-            }
+            JN_TRY(stage<K>(c, s, hc, &x.R, k >= 2, &cr[k][j]));
+            JN_TRY(stage<K>(c, s, hc, &x.S, k >= 2, &cs[k][j]));
+            bops[k].push_back(x.op);
+            bbands[k].push_back(x.band);
         }
     }
     JN_TRY(hc.start());
     JN_TRY(wait_copies(c, true));
     // every join is counted before the single output allocation
-    std::unique_ptr<BatchRun> run[3];
+    std::unique_ptr<BatchRun> run[PARTS];
+    auto move_join = [&](int from, int to, size_t j) {
+        part[to].push_back(part[from][j]);
+        cr[to].push_back(cr[from][j]);
+        cs[to].push_back(cs[from][j]);
+        bops[to].push_back(bops[from][j]);
+        bbands[to].push_back(bbands[from][j]);
+    };
     if (!part[0].empty()) {
         const jn_status st =
             batch_direct_prepare<K>(c, (int)part[0].size(), cr[0].data(), cs[0].data(), count_only, &run[0]);
         if (st == JN_ERR_OOM) {
             // a device too full for the tables and the pairs' room: all of them partitioned
             c->err.clear();
-            for (size_t j = 0; j < part[0].size(); j++) {
-                part[1].push_back(part[0][j]);
-                cr[1].push_back(cr[0][j]);
-                cs[1].push_back(cs[0][j]);
-            }
+            for (size_t j = 0; j < part[0].size(); j++) move_join(0, 1, j);
             part[0].clear();
         } else if (st != JN_OK) {
             return st;
@@ -288,15 +293,35 @@ static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair
     }
     if (!part[1].empty())
         JN_TRY(batch_hash_prepare<K>(c, (int)part[1].size(), cr[1].data(), cs[1].data(), &run[1]));
-    if (!part[2].empty())
-        JN_TRY(batch_band_prepare<K>(c, (int)part[2].size(), cr[2].data(), cs[2].data(), bops.data(), bbands.data(),
-                                     &run[2]));
+    std::vector<char> moved(part[2].size(), 0);  // band joins left to the partitioned join
+    if (!part[2].empty()) {
+        std::unique_ptr<BandDirect> direct;
+        const jn_status st =
+            band_direct_prepare<K>(c, (int)part[2].size(), cr[2].data(), cs[2].data(), bops[2].data(),
+                                   bbands[2].data(), count_only ? MODE_COUNT : MODE_EMIT, &direct);
+        if (st != JN_OK && st != JN_ERR_OOM) return st;
+        c->err.clear();
+        if (st == JN_OK) {
+            moved = direct->stopped;
+            c->info.partitions += direct->buckets;
+            c->info.work_items += direct->tiles;
+            run[2] = std::move(direct);
+        } else {
+            moved.assign(part[2].size(), 1);
+        }
+        for (size_t j = 0; j < part[2].size(); j++)
+            if (moved[j]) move_join(2, 3, j);
+    }
+    if (!part[3].empty())
+        JN_TRY(batch_band_prepare<K>(c, (int)part[3].size(), cr[3].data(), cs[3].data(), bops[3].data(),
+                                     bbands[3].data(), &run[3]));
     uint64_t total = 0;
-    for (int k = 0; k < 3; k++) total += run[k] ? run[k]->total : 0;
+    for (int k = 0; k < PARTS; k++) total += run[k] ? run[k]->total : 0;
     auto publish = [&] {
         uint64_t at = 0;
-        for (int k = 0; k < 3; k++) {
+        for (int k = 0; k < PARTS; k++) {
             for (size_t j = 0; j < part[k].size(); j++) {
+                if (k == 2 && moved[j]) continue;
                 first[part[k][j]] = at + run[k]->offsets[j];
                 pairs[part[k][j]] = run[k]->offsets[j + 1] - run[k]->offsets[j];
             }
@@ -317,7 +342,7 @@ static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair
     if (plan.host_copy && !is_device_pointer(*out))
         return fail(c, JN_ERR_INVALID, "batch outputs must be device memory");
     uint64_t at = 0;
-    for (int k = 0; k < 3; k++) {
+    for (int k = 0; k < PARTS; k++) {
         if (!run[k]) continue;
         JN_TRY(run[k]->emit(c, plan.dev + at));
         at += run[k]->total;

@@ -46,6 +46,8 @@ enum KernelId {
     K_STAR,
     K_DIRECT_BUILD,
     K_DIRECT_PROBE,
+    K_BAND_BUILD,
+    K_BAND_PROBE,
     K_COUNT_IDS
 };
 
@@ -179,6 +181,7 @@ jn_status read_back(jn_ctx* c, const uint64_t* dsrc, uint64_t* hdst, int n);
 // Exclusive scan: out[i] = sum(in[0..i-1]) for i in [0, n]; out has n + 1 words.
 jn_status scan_u32(jn_ctx* c, const uint32_t* in, uint64_t* out, int64_t n);
 jn_status scan_u64(jn_ctx* c, const uint64_t* in, uint64_t* out, int64_t n);
+jn_status scan_u32_u32(jn_ctx* c, const uint32_t* in, uint32_t* out, int64_t n);  // sums below 2^32
 
 // Host-side column staging: returns a device pointer for a column that may
 // be host memory (copied into scratch) or device memory (returned as is).

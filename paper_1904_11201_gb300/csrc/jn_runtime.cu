@@ -19,7 +19,7 @@ static const char* kKernelNames[K_COUNT_IDS] = {
     "nlj_emit",     "minmax",       "theta_count", "theta_emit",  "gather",
     "batch",        "misc",         "sort_count",  "sort_emit",   "sort_chunks",
     "chunk_hist",   "region1",      "region2",     "theta_gather", "star",
-    "direct_build", "direct_probe"};
+    "direct_build", "direct_probe", "band_build",  "band_probe"};
 
 const char* kernel_name(int kid) {
     return (kid >= 0 && kid < K_COUNT_IDS) ? kKernelNames[kid] : "?";
@@ -188,8 +188,8 @@ __global__ void k_scan_reduce(const T* __restrict__ in, int64_t n, uint64_t* __r
 // One block scans in[0..n) with a running carry; out[n] = total.  With
 // `carry_in` != nullptr, each block's carry comes from carry_in[blockIdx.x]
 // (the down-sweep over chunks of SCAN_CHUNK).
-template <typename T>
-__global__ void k_scan_chunks(const T* __restrict__ in, int64_t n, uint64_t* __restrict__ out,
+template <typename T, typename O>
+__global__ void k_scan_chunks(const T* __restrict__ in, int64_t n, O* __restrict__ out,
                               const uint64_t* __restrict__ carry_in) {
     __shared__ uint64_t tmp[33];
     uint64_t carry = carry_in ? carry_in[blockIdx.x] : 0;
@@ -209,18 +209,18 @@ __global__ void k_scan_chunks(const T* __restrict__ in, int64_t n, uint64_t* __r
 #pragma unroll
         for (int j = 0; j < SCAN_V; j++) {
             int64_t i = base + (int64_t)threadIdx.x * SCAN_V + j;
-            if (i < end) out[i] = pre;
+            if (i < end) out[i] = (O)pre;
             pre += v[j];
         }
         carry += total;
     }
-    if (threadIdx.x == 0 && end == n) out[n] = carry;
+    if (threadIdx.x == 0 && end == n) out[n] = (O)carry;
 }
 
-template <typename T>
-static jn_status scan_impl(jn_ctx* c, const T* in, uint64_t* out, int64_t n) {
+template <typename T, typename O>
+static jn_status scan_impl(jn_ctx* c, const T* in, O* out, int64_t n) {
     if (n <= 8 * SCAN_CHUNK) {
-        return launch(c, K_SCAN_TOP, k_scan_chunks<T>, dim3(1), dim3(SCAN_T), 0, in, n, out,
+        return launch(c, K_SCAN_TOP, (k_scan_chunks<T, O>), dim3(1), dim3(SCAN_T), 0, in, n, out,
                       (const uint64_t*)nullptr);
     }
     int64_t nb = (int64_t)ceil_div(n, SCAN_CHUNK);
@@ -230,17 +230,20 @@ static jn_status scan_impl(jn_ctx* c, const T* in, uint64_t* out, int64_t n) {
     JN_TRY(s.get(&pre, nb + 1));
     JN_TRY(launch(c, K_SCAN_REDUCE, k_scan_reduce<T>, dim3((unsigned)nb), dim3(SCAN_T), 0, in, n,
                   sums));
-    JN_TRY(scan_impl<uint64_t>(c, sums, pre, nb));
-    JN_TRY(launch(c, K_SCAN_DOWN, k_scan_chunks<T>, dim3((unsigned)nb), dim3(SCAN_T), 0, in, n,
+    JN_TRY((scan_impl<uint64_t, uint64_t>(c, sums, pre, nb)));
+    JN_TRY(launch(c, K_SCAN_DOWN, (k_scan_chunks<T, O>), dim3((unsigned)nb), dim3(SCAN_T), 0, in, n,
                   out, (const uint64_t*)pre));
     return JN_OK;
 }
 
 jn_status scan_u32(jn_ctx* c, const uint32_t* in, uint64_t* out, int64_t n) {
-    return scan_impl<uint32_t>(c, in, out, n);
+    return scan_impl<uint32_t, uint64_t>(c, in, out, n);
+}
+jn_status scan_u32_u32(jn_ctx* c, const uint32_t* in, uint32_t* out, int64_t n) {
+    return scan_impl<uint32_t, uint32_t>(c, in, out, n);
 }
 jn_status scan_u64(jn_ctx* c, const uint64_t* in, uint64_t* out, int64_t n) {
-    return scan_impl<uint64_t>(c, in, out, n);
+    return scan_impl<uint64_t, uint64_t>(c, in, out, n);
 }
 
 }  // namespace jnx

@@ -96,11 +96,6 @@ __global__ void __launch_bounds__(512) k_minmax(const K* __restrict__ col, int64
     }
 }
 
-__global__ void k_mm_init(long long* mm) {
-    mm[0] = LLONG_MAX;
-    mm[1] = LLONG_MIN;
-}
-
 // Group width 2^shift: the smallest power of two with (hi - lo) >> shift < G.
 __global__ void k_range_setup(const long long* __restrict__ mm, int G, RangeParams* __restrict__ p) {
     long long lo = mm[0], hi = mm[1];
@@ -151,12 +146,6 @@ struct ThetaSet {
     const int* groups;
     int lg;
 };
-
-__global__ void k_set_theta_one(long long* band, int* op, int* groups, long long b, int o, int g) {
-    *band = b;
-    *op = o;
-    *groups = g;
-}
 
 // items[p] = R chunks of the window of group y of its join x S chunks of y.
 // With `bound`, adds sum_y |window of y| * |S_y| to it: the pairs the
@@ -631,45 +620,27 @@ k_cross_emit(const R* __restrict__ rrows, const uint64_t* __restrict__ roff, con
     }
 }
 
-template <typename K, bool HB>
-static jn_status range_partition(jn_ctx* c, Scratch& s, const Cols<K>& T, const K* grp, const K* carry,
-                                 const RangeParams* prm, int G, unsigned int* work, Row<K, HB>** orows,
-                                 uint64_t** off) {
-    const uint64_t n = (uint64_t)T.n;
-    uint64_t *sb, *scn, *tp, *start;
-    unsigned long long *hist, *cur;
-    JN_TRY(s.get(&sb, 2));
-    JN_TRY(s.get(&scn, 2));
-    JN_TRY(s.get(&tp, 3));
-    JN_TRY(s.get(&start, G + 1));
-    JN_TRY(s.get(&hist, G));
-    JN_TRY(s.get(&cur, G));
-    JN_TRY(zero(c, hist, sizeof(unsigned long long) * G));
-    JN_TRY(launch(c, K_SEGMENTS, k_one_segment, dim3(1), dim3(32), 0, sb, scn, tp, n));
-    RangeDigit dg{prm};
-    auto kh = k_seg_hist<K, RangeDigit>;
-    const size_t smh = sizeof(uint32_t) * G;
-    int per = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kh, SC_T, smh);
-    JN_TRY(launch(c, K_HIST, kh, dim3(max(per, 1) * c->num_sms), dim3(SC_T), smh, grp,
-                  (const uint64_t*)sb, (const uint64_t*)scn, (const uint64_t*)tp, 1, dg, G, hist, work));
-    JN_TRY(scan_u64(c, reinterpret_cast<const uint64_t*>(hist), start, G));
-    JN_TRY(launch(c, K_MISC, k_init_cursor, dim3((G + 255) / 256), dim3(256), 0, (const uint64_t*)start,
-                  cur, (int64_t)G));
-    Row<K, HB>* rows;
-    JN_TRY(s.get(&rows, n + 16));
-    auto ks = k_scatter<K, HB, false, RangeDigit>;
-    const size_t sm = scatter_smem<K, HB>();
-    per = 0;
-    ensure_smem((const void*)ks, sm);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ks, SC_T, sm);
-    PartIn<K, HB> in{grp, carry, T.pay, nullptr, n, nullptr, nullptr};
-    JN_TRY(launch(c, K_SCATTER, ks, dim3(max(per, 1) * c->num_sms), dim3(SC_T), sm, in, (const uint64_t*)sb,
-                  (const uint64_t*)scn, (const uint64_t*)tp, 1, dg, G, (const uint32_t*)nullptr, 0u, cur, rows,
-                  c->d_err));
-    *orows = rows;
-    *off = start;
-    return JN_OK;
+// What a single join's kernels expect to find: the range's empty bounds, the
+// join's predicate, and each table as one segment of its range pass.
+struct ThetaOne {
+    long long mm[2];
+    long long band;
+    int op, groups;
+    uint64_t seg_begin, rcount, scount;
+    uint64_t rtiles[2], stiles[2];  // tile prefixes
+};
+__global__ void k_theta_one(ThetaOne* t, long long band, int op, int groups, uint64_t nr, uint64_t ns) {
+    t->mm[0] = LLONG_MAX;
+    t->mm[1] = LLONG_MIN;
+    t->band = band;
+    t->op = op;
+    t->groups = groups;
+    t->seg_begin = 0;
+    t->rcount = nr;
+    t->scount = ns;
+    t->rtiles[0] = t->stiles[0] = 0;
+    t->rtiles[1] = (nr + SC_TILE - 1) / SC_TILE;
+    t->stiles[1] = (ns + SC_TILE - 1) / SC_TILE;
 }
 
 template <typename K, bool B>
@@ -685,35 +656,61 @@ static jn_status run_theta_t(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int 
         if (g > 10) g = 10;
     }
     const int G = 1 << g;
+    const uint64_t nr = (uint64_t)R.n, ns = (uint64_t)S.n;
     Scratch s(c);
-    unsigned int* work;
-    long long* mm;
+    // one block of words that start as zeros: small results, the checksum, the
+    // work counters of three kernels, the histograms of R's and S's groups
+    uint64_t *zeroed, *start;
+    ThetaOne* one;
     RangeParams* prm;
-    uint64_t* d_small;
-    JN_TRY(s.get(&work, 4));
-    JN_TRY(s.get(&mm, 2));
+    unsigned long long* cur;
+    RW* rows;  // R's rows, then S's, each grouped
+    JN_TRY(s.get(&zeroed, (size_t)8 + 2 * G));
+    JN_TRY(s.get(&one, 1));
     JN_TRY(s.get(&prm, 1));
-    JN_TRY(s.get(&d_small, 4));
-    JN_TRY(zero(c, d_small, 4 * sizeof(uint64_t)));
+    JN_TRY(s.get(&start, 2 * (size_t)G + 1));
+    JN_TRY(s.get(&cur, 2 * (size_t)G));
+    JN_TRY(s.get(&rows, nr + ns + 16));
+    JN_TRY(zero(c, zeroed, 8 * (8 + 2 * (size_t)G)));
+    uint64_t* d_small = zeroed;
+    unsigned long long* chk = reinterpret_cast<unsigned long long*>(zeroed + 4);
+    unsigned int* work = reinterpret_cast<unsigned int*>(zeroed + 5);  // [0] count, [1] emit, [2] cross regions
+    unsigned long long* hist = reinterpret_cast<unsigned long long*>(zeroed + 8);
     const K* rg = B ? R.key2 : R.key;
     const K* sg = B ? S.key2 : S.key;
-    JN_TRY(launch(c, K_MINMAX, k_mm_init, dim3(1), dim3(1), 0, mm));
-    JN_TRY(launch(c, K_MINMAX, k_minmax<K>, dim3(2 * c->num_sms), dim3(512), 0, rg, R.n, mm));
-    JN_TRY(launch(c, K_MINMAX, k_minmax<K>, dim3(2 * c->num_sms), dim3(512), 0, sg, S.n, mm));
-    JN_TRY(launch(c, K_MINMAX, k_range_setup, dim3(1), dim3(1), 0, (const long long*)mm, G, prm));
-    RW *rrows, *srows;
-    uint64_t *roff, *soff;
-    JN_TRY((range_partition<K, B>(c, s, R, rg, B ? R.key : nullptr, prm, G, work, &rrows, &roff)));
-    JN_TRY((range_partition<K, B>(c, s, S, sg, B ? S.key : nullptr, prm, G, work, &srows, &soff)));
+    JN_TRY(launch(c, K_MINMAX, k_theta_one, dim3(1), dim3(1), 0, one, (long long)(B ? band : -1), op, G, nr, ns));
+    JN_TRY(launch(c, K_MINMAX, k_minmax<K>, dim3(2 * c->num_sms), dim3(512), 0, rg, R.n, one->mm));
+    JN_TRY(launch(c, K_MINMAX, k_minmax<K>, dim3(2 * c->num_sms), dim3(512), 0, sg, S.n, one->mm));
+    JN_TRY(launch(c, K_MINMAX, k_range_setup, dim3(1), dim3(1), 0, (const long long*)one->mm, G, prm));
+    // ---- range partition of both tables ----
+    RangeDigit dg{prm};
+    auto kh = k_seg_hist<K, RangeDigit>;
+    auto ks = k_scatter<K, B, false, RangeDigit>;
+    const size_t smh = sizeof(uint32_t) * G, sms = scatter_smem<K, B>();
+    int perh = 0, pers = 0;
+    ensure_smem((const void*)ks, sms);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perh, kh, SC_T, smh);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pers, ks, SC_T, sms);
+    const dim3 gh(max(perh, 1) * c->num_sms), gs(max(pers, 1) * c->num_sms);
+    JN_TRY(launch(c, K_HIST, kh, gh, dim3(SC_T), smh, rg, (const uint64_t*)&one->seg_begin,
+                  (const uint64_t*)&one->rcount, (const uint64_t*)one->rtiles, 1, dg, G, hist, work));
+    JN_TRY(launch(c, K_HIST, kh, gh, dim3(SC_T), smh, sg, (const uint64_t*)&one->seg_begin,
+                  (const uint64_t*)&one->scount, (const uint64_t*)one->stiles, 1, dg, G, hist + G, work));
+    JN_TRY(scan_u64(c, reinterpret_cast<const uint64_t*>(hist), start, 2 * (int64_t)G));
+    JN_TRY(launch(c, K_MISC, k_init_cursor, dim3((2 * G + 255) / 256), dim3(256), 0, (const uint64_t*)start, cur,
+                  2 * (int64_t)G));
+    PartIn<K, B> inr{rg, B ? R.key : nullptr, R.pay, nullptr, nr, nullptr, nullptr};
+    PartIn<K, B> ins{sg, B ? S.key : nullptr, S.pay, nullptr, ns, nullptr, nullptr};
+    JN_TRY(launch(c, K_SCATTER, ks, gs, dim3(SC_T), sms, inr, (const uint64_t*)&one->seg_begin,
+                  (const uint64_t*)&one->rcount, (const uint64_t*)one->rtiles, 1, dg, G, (const uint32_t*)nullptr, 0u,
+                  cur, rows, c->d_err));
+    JN_TRY(launch(c, K_SCATTER, ks, gs, dim3(SC_T), sms, ins, (const uint64_t*)&one->seg_begin,
+                  (const uint64_t*)&one->scount, (const uint64_t*)one->stiles, 1, dg, G, (const uint32_t*)nullptr, 0u,
+                  cur + G, rows, c->d_err));
+    RW *rrows = rows, *srows = rows;
+    const uint64_t *roff = start, *soff = start + G;
     // ---- compared regions (band window or diagonal) ----
-    long long* d_band;
-    int *d_op, *d_groups;
-    JN_TRY(s.get(&d_band, 1));
-    JN_TRY(s.get(&d_op, 2));
-    d_groups = d_op + 1;
-    JN_TRY(launch(c, K_MISC, k_set_theta_one, dim3(1), dim3(1), 0, d_band, d_op, d_groups,
-                  (long long)(B ? band : -1), op, G));
-    const ThetaSet ts{prm, d_band, d_op, d_groups, g};
+    const ThetaSet ts{prm, &one->band, &one->op, &one->groups, g};
     uint64_t *items, *ipre;
     JN_TRY(s.get(&items, G));
     JN_TRY(s.get(&ipre, G + 1));
@@ -737,12 +734,10 @@ static jn_status run_theta_t(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int 
     uint64_t h0[4];
     JN_TRY(read_back(c, d_small, h0, 4));
     const uint64_t nitems = h0[0], compared = h0[3];
-    unsigned long long *ival, *chk;
+    unsigned long long* ival;
     uint64_t* ioff;
     JN_TRY(s.get(&ival, nitems + 1));
     JN_TRY(s.get(&ioff, nitems + 1));
-    JN_TRY(s.get(&chk, 1));
-    JN_TRY(zero(c, chk, 8));
     const int cm = mode == MODE_AGG ? MODE_AGG : MODE_COUNT;
     auto pick = [&](int m) {
         if (m == MODE_EMIT) return k_theta_join<K, MODE_EMIT, B>;
@@ -764,13 +759,11 @@ static jn_status run_theta_t(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int 
         JN_TRY(s.get(&rec.pay, nitems * TH_RCAP));
         JN_TRY(s.get(&rec.sdesc, nitems));
         rec.any_wide = reinterpret_cast<unsigned int*>(d_small + 2);
-        JN_TRY(zero(c, d_small + 2, 8));
         // the gather reads the saved payloads as 16-byte words
         if ((uintptr_t)rec.pay & 15) rec = ThetaRec{nullptr, nullptr, nullptr, nullptr};
     }
     if (nitems) {
         auto kc = pick(cm);
-        JN_TRY(zero(c, work, 4));
         JN_TRY(launch(c, K_THETA_COUNT, kc, dim3(grid_of((const void*)kc, theta_smem<K>(cm))), dim3(TH_T),
                       theta_smem<K>(cm), (const RW*)rrows,
                       (const uint64_t*)roff, (const RW*)srows, (const uint64_t*)soff, ts, G, (const uint64_t*)ipre,
@@ -815,18 +808,16 @@ static jn_status run_theta_t(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int 
     if (diag && (!rec.rows || any_wide)) {
         // every item, or (after the gather) the wide ones
         auto ke = pick(MODE_EMIT);
-        JN_TRY(zero(c, work, 4));
         JN_TRY(launch(c, K_THETA_EMIT, ke, dim3(grid_of((const void*)ke, theta_smem<K>(MODE_EMIT))), dim3(TH_T),
                       theta_smem<K>(MODE_EMIT), (const RW*)rrows,
                       (const uint64_t*)roff, (const RW*)srows, (const uint64_t*)soff, ts, G, (const uint64_t*)ipre,
                       (unsigned long long*)nullptr, (unsigned long long*)nullptr, (const uint64_t*)ioff, plan->dev,
-                      work, rec));
+                      work + 1, rec));
     }
     if (crossn) {
-        JN_TRY(zero(c, work, 4));
         JN_TRY(launch(c, K_CROSS_EMIT, k_cross_emit<RW>, dim3(4 * c->num_sms), dim3(256), 0, (const RW*)rrows,
                       (const uint64_t*)roff, (const RW*)srows, (const uint64_t*)soff, (const uint64_t*)coff,
-                      (const uint64_t*)cpre, G, op, diag, plan->dev, work));
+                      (const uint64_t*)cpre, G, op, diag, plan->dev, work + 2));
     }
     JN_TRY(out_finish(c, total, *plan));
     return JN_OK;
@@ -843,6 +834,27 @@ jn_status run_theta(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int op, int64
             JN_TRY(out_finish(c, 0, *plan));
         }
         return JN_OK;
+    }
+    if (band >= 0 && band_direct_takes(c, R.n, S.n)) {
+        std::unique_ptr<BandDirect> run;
+        const jn_status st = band_direct_prepare<K>(c, 1, &R, &S, &op, &band, mode, &run);
+        if (st == JN_OK && !run->stopped[0]) {
+            jn_run_info& info = c->info;
+            res->count = info.result = run->total;
+            res->checksum = run->checksum;
+            info.partitions = run->buckets;
+            info.work_items = run->tiles;
+            info.r_survivors = (uint64_t)R.n;
+            info.s_survivors = (uint64_t)S.n;
+            info.cartesian_bound = run->candidates;
+            if (mode != MODE_EMIT) return JN_OK;
+            Scratch s(c);
+            JN_TRY(out_prepare(c, s, run->total, *plan));
+            JN_TRY(run->emit(c, plan->dev));
+            return out_finish(c, run->total, *plan);
+        }
+        if (st != JN_OK && st != JN_ERR_OOM) return st;
+        c->err.clear();  // too full a device or too many candidates: partitioned
     }
     if (band >= 0) return run_theta_t<K, true>(c, R, S, op, band, mode, plan, res);
     return run_theta_t<K, false>(c, R, S, op, band, mode, plan, res);
