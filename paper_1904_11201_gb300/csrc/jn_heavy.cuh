@@ -17,7 +17,6 @@ namespace jnx {
 
 constexpr int HV_MAX = 1024;         // heavy keys at most (digits of the heavy grouping pass)
 constexpr int HV_SLOTS = 4096;       // open-addressing table of heavy keys
-constexpr int HV_FBITS = 16;         // shared-memory filter of 2^16 bits over khash
 constexpr int HV_SAMPLE_LOG = 21;    // sample table slots (log2)
 
 template <typename K>
@@ -48,25 +47,28 @@ __device__ __forceinline__ int hv_lookup(const HeavySet<K>& hs, K k) {
     return -1;
 }
 
-// Fills the shared-memory filter (2^HV_FBITS bits, HV_FBITS / 8 KB) from the
-// heavy list; all threads of the block call it, followed by __syncthreads.
+// The heavy keys alone as a table in shared memory (HV_SLOTS keys, the
+// sentinel key in the empty slots): whether a row is set aside takes one or two
+// shared reads.  A filter in shared memory with the table behind it in global
+// memory made every heavy row, most of a skewed column, look there.  All
+// threads of the block call it, followed by __syncthreads.
 template <typename K>
-__device__ __forceinline__ void hv_filter_fill(uint32_t* f, const HeavySet<K>& hs) {
-    for (int i = threadIdx.x; i < (1 << HV_FBITS) / 32; i += blockDim.x) f[i] = 0;
-    __syncthreads();
-    const int h = *hs.count;
-    for (int i = threadIdx.x; i < h; i += blockDim.x) {
-        const uint32_t b = khash(hs.keys[i]) >> (32 - HV_FBITS);
-        atomicOr(&f[b >> 5], 1u << (b & 31));
-    }
+__device__ __forceinline__ void hv_member_fill(K* t, const HeavySet<K>& hs) {
+    for (int i = threadIdx.x; i < HV_SLOTS; i += blockDim.x)
+        t[i] = hs.tab_idx[i] >= 0 ? hs.tab_key[i] : key_sentinel<K>();
 }
 
-// Index of k in the heavy set, or -1; the filter answers most misses.
+// Whether k is heavy (the sentinel key never is).
 template <typename K>
-__device__ __forceinline__ int hv_find(const uint32_t* f, const HeavySet<K>& hs, K k) {
-    const uint32_t b = khash(k) >> (32 - HV_FBITS);
-    if (!((f[b >> 5] >> (b & 31)) & 1u)) return -1;
-    return hv_lookup(hs, k);
+__device__ __forceinline__ bool hv_member(const K* t, K k) {
+    uint32_t s = hv_slot(khash(k));
+    for (int probe = 0; probe < HV_SLOTS; probe++) {
+        const K x = t[s];
+        if (x == key_sentinel<K>()) return false;
+        if (x == k) return true;
+        s = (s + 1) & (HV_SLOTS - 1);
+    }
+    return false;
 }
 
 // ------------------------------------------------------------- sampling --
@@ -176,22 +178,27 @@ __global__ void k_heavy_collect(const K* __restrict__ tk, const unsigned int* __
     }
 }
 
-// One block: caps the heavy count and builds the key -> index table.
+// One block: caps the heavy count and builds the key -> index table, put
+// together in shared memory by all threads (one thread inserting into global
+// memory took 0.25 ms for 1000 keys).
 template <typename K>
 __global__ void k_heavy_table(const K* __restrict__ keys, K* __restrict__ tab_key, int* __restrict__ tab_idx,
                               int* __restrict__ count) {
-    for (int i = threadIdx.x; i < HV_SLOTS; i += blockDim.x) tab_idx[i] = -1;
+    __shared__ int s_idx[HV_SLOTS];
+    for (int i = threadIdx.x; i < HV_SLOTS; i += blockDim.x) s_idx[i] = -1;
+    const int h = min(*count, HV_MAX);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const int h = *count < HV_MAX ? *count : HV_MAX;
-        for (int i = 0; i < h; i++) {
-            uint32_t s = hv_slot(khash(keys[i]));
-            while (tab_idx[s] >= 0) s = (s + 1) & (HV_SLOTS - 1);
-            tab_key[s] = keys[i];
-            tab_idx[s] = i;
-        }
-        *count = h;
+    for (int i = threadIdx.x; i < h; i += blockDim.x) {  // the keys are distinct
+        uint32_t s = hv_slot(khash(keys[i]));
+        while (atomicCAS(&s_idx[s], -1, i) != -1) s = (s + 1) & (HV_SLOTS - 1);
     }
+    __syncthreads();
+    for (int s = threadIdx.x; s < HV_SLOTS; s += blockDim.x) {
+        const int i = s_idx[s];
+        tab_idx[s] = i;
+        if (i >= 0) tab_key[s] = keys[i];
+    }
+    if (threadIdx.x == 0) *count = h;
 }
 
 // Sets the presence bit of every heavy key (the presence kernel skips
@@ -220,27 +227,89 @@ struct HeavyIdxDigit {
 };
 
 // Digit of pass 1 with heavy keys set aside: F1 for a heavy key, else the
-// hash digit.  `f` is the block's shared-memory filter.
+// hash digit.  `t` is the block's table of the heavy keys.
 template <typename K>
 struct HeavyHashDigit {
-    static constexpr int kFilterWords = (1 << HV_FBITS) / 32;
+    static constexpr int kFilterWords = HV_SLOTS * (int)sizeof(K) / 4;
     int shift;
     uint32_t mask;
     uint32_t heavy_digit;
     HeavySet<K> hs;
-    const uint32_t* f;
+    const K* t;
     __device__ __forceinline__ bool is_special(uint32_t d) const { return d == heavy_digit; }
     __device__ __forceinline__ void set_seg(int) {}
-    // Fills the block's filter; all threads call it (it synchronises).
-    __device__ __forceinline__ void bind(uint32_t* smem_filter) {
-        hv_filter_fill(smem_filter, hs);
+    // Fills the block's table; all threads call it (it synchronises).
+    __device__ __forceinline__ void bind(uint32_t* smem) {
+        K* m = reinterpret_cast<K*>(smem);
+        hv_member_fill(m, hs);
         __syncthreads();
-        f = smem_filter;
+        t = m;
     }
     __device__ __forceinline__ uint32_t operator()(K k) const {
-        return hv_find(f, hs, k) >= 0 ? heavy_digit : ((khash(k) >> shift) & mask);
+        return hv_member(t, k) ? heavy_digit : ((khash(k) >> shift) & mask);
     }
 };
+
+// ------------------------------------------------------ counts and sums --
+// What a count or a checksum needs of a table's heavy rows: per heavy key, its
+// rows and (with_sum) the sum of f over them (g when use_g), added to cnt[] and
+// sum[].  Rows [seg[0], seg[1]) of `rows`, in any order: nothing is grouped.
+template <typename K>
+__global__ void __launch_bounds__(512)
+k_heavy_sums(const Row<K, false>* __restrict__ rows, const uint64_t* __restrict__ seg, HeavySet<K> hs, int use_g,
+             int with_sum, unsigned long long* __restrict__ cnt, unsigned long long* __restrict__ sum) {
+    __shared__ uint32_t s_cnt[HV_MAX], s_lo[HV_MAX], s_hi[HV_MAX];
+    for (int i = threadIdx.x; i < HV_MAX; i += blockDim.x) s_cnt[i] = s_lo[i] = s_hi[i] = 0;
+    __syncthreads();
+    const uint64_t end = seg[1], stride = (uint64_t)gridDim.x * blockDim.x;
+    uint32_t taken = 0;
+    // a block adds fewer than 2^32 rows: its counts and carries fit
+    for (uint64_t i = seg[0] + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end; i += 4 * stride) {
+        Row<K, false> x[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (i + u * stride < end) x[u] = rows[i + u * stride];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (i + u * stride >= end) continue;
+            const int h = hv_lookup(hs, x[u].key);
+            if (h < 0) continue;
+            taken++;
+            atomicAdd(&s_cnt[h], 1u);
+            if (!with_sum) continue;
+            // a 64-bit sum in two native adds: the low word tells its carry
+            const unsigned long long f = use_g ? chk_g(x[u].pay) : chk_f(x[u].pay);
+            const uint32_t w = (uint32_t)f, o = atomicAdd(&s_lo[h], w);
+            atomicAdd(&s_hi[h], (uint32_t)(f >> 32) + (o + w < o ? 1u : 0u));
+        }
+    }
+    if (!__syncthreads_or(taken != 0)) return;
+    for (int i = threadIdx.x; i < HV_MAX; i += blockDim.x) {
+        if (!s_cnt[i]) continue;
+        atomicAdd(&cnt[i], (unsigned long long)s_cnt[i]);
+        if (with_sum) atomicAdd(&sum[i], (unsigned long long)s_hi[i] << 32 | s_lo[i]);
+    }
+}
+
+// One block: *total = sum over heavy keys of rows in R * rows in S, and *chk +=
+// the sum of fsum * gsum.
+static __global__ void k_heavy_totals(const unsigned long long* __restrict__ cr, const unsigned long long* __restrict__ cs,
+                                      const unsigned long long* __restrict__ fsum,
+                                      const unsigned long long* __restrict__ gsum, uint64_t* __restrict__ total,
+                                      unsigned long long* __restrict__ chk) {
+    __shared__ unsigned long long tmp[33];
+    unsigned long long n = 0, v = 0;
+    for (int h = threadIdx.x; h < HV_MAX; h += blockDim.x) {
+        n += cr[h] * cs[h];
+        v += fsum[h] * gsum[h];
+    }
+    n = block_sum(n, tmp);
+    v = block_sum(v, tmp);
+    if (threadIdx.x == 0) {
+        *total = n;
+        if (v) atomicAdd(chk, v);
+    }
+}
 
 // ---------------------------------------------------------- cross product --
 // Per heavy key h: pairs c_R(h) * c_S(h) (block x = 0 writes them) and, for

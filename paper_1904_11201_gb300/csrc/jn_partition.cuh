@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(512)
 k_presence_hist(const K* __restrict__ keys, int64_t n, uint32_t* __restrict__ bitmap,
                 uint32_t fmask, Digit dg0, int nd, unsigned long long* __restrict__ hist) {
     extern __shared__ uint32_t s_h[];
-    __shared__ uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
+    __shared__ __align__(8) uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
     Digit dg = dg0;
     dg.bind(s_dgf);
     if (hist)
@@ -232,7 +232,7 @@ k_seg_hist(const K* __restrict__ keys, const uint64_t* __restrict__ seg_begin,
            unsigned int* __restrict__ work) {
     extern __shared__ uint32_t s_h[];
     __shared__ uint64_t s_tp[SC_FMAX + 1];
-    __shared__ uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
+    __shared__ __align__(8) uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
     Digit dg = dg0;
     dg.bind(s_dgf);
     for (int i = threadIdx.x; i <= nseg; i += blockDim.x) s_tp[i] = tile_prefix[i];
@@ -303,7 +303,7 @@ k_seg_hist_rows(const R* __restrict__ rows, const uint64_t* __restrict__ seg_beg
                 Digit dg0, int nd, unsigned long long* __restrict__ hist) {
     extern __shared__ uint32_t s_h[];
     __shared__ uint64_t s_tp[SC_FMAX + 1];
-    __shared__ uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
+    __shared__ __align__(8) uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
     Digit dg = dg0;
     dg.bind(s_dgf);
     for (int i = threadIdx.x; i <= nseg; i += blockDim.x) s_tp[i] = tile_prefix[i];
@@ -478,7 +478,7 @@ k_scatter(PartIn<K, HB> in, const uint64_t* __restrict__ seg_begin, const uint64
     __shared__ TileDesc desc[2];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint64_t s_tp[SC_FMAX + 1];
-    __shared__ uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
+    __shared__ __align__(8) uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
     Digit dg = dg0;
     dg.bind(s_dgf);
 

@@ -1,6 +1,5 @@
 // Join of one hash partition pair in shared memory (the join kernel of the
-// partitioned hash join, for inputs without many frequent keys; k_hash_join
-// serves the others).
+// partitioned hash join).
 //
 // A work item is a chunk of R rows of one partition against every S row of
 // that partition.  The R rows are staged in shared memory (one TMA bulk copy)

@@ -85,7 +85,7 @@ template <typename K, typename Digit>
 __global__ void __launch_bounds__(512)
 k_chunk_hist(const K* __restrict__ keys, int64_t n, int64_t chunk, Digit dg0, int nd, uint32_t* __restrict__ hist) {
     extern __shared__ uint32_t s_h[];
-    __shared__ uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
+    __shared__ __align__(8) uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
     Digit dg = dg0;
     dg.bind(s_dgf);
     constexpr int V = 16 / (int)sizeof(K);
@@ -237,7 +237,7 @@ k_region1_scatter(const K* __restrict__ key, const int32_t* __restrict__ pay, in
     __shared__ uint32_t s_wsum[32];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ StageTile tile[2];
-    __shared__ uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
+    __shared__ __align__(8) uint32_t s_dgf[Digit::kFilterWords > 0 ? Digit::kFilterWords : 1];
     Digit dg = dg0;
     dg.bind(s_dgf);
     const int tid = threadIdx.x;

@@ -15,9 +15,8 @@
 //      hash table on the R chunk, probes it with the partition's S rows and
 //      keeps the pairs it finds in scratch (jn_partjoin.cuh).
 //   5. one exact allocation (the total is one 8-byte read-back) and one copy.
-//      Inputs with many frequent keys, and the sort-merge join, count per item
-//      in step 4, scan the counts to output offsets, and join a second time to
-//      write the pairs there.
+//      The sort-merge join counts per item in step 4, scans the counts to
+//      output offsets, and joins a second time to write the pairs there.
 #include <vector>
 
 #include "jn_algos.h"
@@ -137,12 +136,11 @@ struct alignas(2 * sizeof(K)) RunSlot {
     uint32_t packed;
 };
 
-// Shared-memory layout of the join kernel (bytes), shared by host and device,
-// for a table of CAP_ R rows.
-template <typename K, int MODE, int CAP_ = cap_of<K>()>
+// Shared-memory layout of the batch join kernel (bytes), shared by host and device.
+template <typename K, int MODE>
 struct JoinSmem {
     using R = Row<K, false>;
-    static constexpr int CAP = CAP_;
+    static constexpr int CAP = cap_of<K>();
     static constexpr int GR = CAP + 32 / (int)sizeof(R) + 2;     // staged R rows (widened span)
     static constexpr int GS = HJ_SCH + 32 / (int)sizeof(R) + 2;  // staged S rows per buffer
     static constexpr int TS = (CAP * 5) / 4;                     // open-addressing slots
@@ -150,7 +148,7 @@ struct JoinSmem {
     // emit: TS slots and one for the sentinel key, then the payloads grouped by slot
     static constexpr size_t TABLE =
         MODE == MODE_EMIT ? (size_t)(TS + 1) * sizeof(RunSlot<K>) + (size_t)CAP * 4
-                          : (size_t)TS * (sizeof(K) + 4) + (MODE == MODE_AGG ? (size_t)TS * 8 : 0);
+                          : (size_t)TS * (sizeof(K) + 4);
     static constexpr size_t BYTES = STAGE + TABLE;
 };
 static_assert(cap_of<int32_t>() < (1 << 16), "run cursors and counts fit half a word");
@@ -162,10 +160,9 @@ __device__ __forceinline__ uint32_t oa_slot(uint32_t h, int bits, int ts) {
     return (uint32_t)(((uint64_t)x * (uint64_t)ts) >> 32);
 }
 
-// The join kernel of inputs with many frequent keys (MERGE) and of batches;
-// the others take k_part_join.
+// The join kernel of batches' partitioned equi-joins, whose items count before
+// they write (single joins take k_part_join).
 // MODE_COUNT: item_val[it] = matches of the item.
-// MODE_AGG:   as COUNT, and chk += sum over matches of f(r) * g(s).
 // MODE_EMIT:  writes the item's pairs at out[item_off[it] ...].
 //
 // Items (a chunk of R rows of one partition against all S rows of that
@@ -176,24 +173,22 @@ __device__ __forceinline__ uint32_t oa_slot(uint32_t h, int bits, int ts) {
 //   emit:         each distinct R key gets one slot holding its multiplicity
 //                 and the run of its payloads in a slot-grouped array, so a
 //                 match is one lookup and a contiguous copy;
-//   count / agg:  equal R keys are folded into one open-addressing slot
-//                 (key, multiplicity [, sum of f]), so a probe costs one
-//                 lookup however many rows share the key.
+//   count:        equal R keys are folded into one open-addressing slot
+//                 (key, multiplicity), so a probe costs one lookup however
+//                 many rows share the key.
 // The partitioned rows are library scratch, 16-byte aligned and padded by
 // HJ_PAD rows, so every widened copy stays inside its allocation.
 // PU: S rows a thread probes per round.  The emit pass overlaps HJ_PU rows'
 // lookups and reserves their output once; the count pass, with no output to
 // reserve, measured fastest with one.
-template <typename K, int MODE, bool MERGE = false, int CAP = cap_of<K>(), int PU = (MODE == MODE_EMIT ? HJ_PU : 1)>
-__global__ void __launch_bounds__(HJ_T, (CAP < cap_of<K>() && MODE != MODE_EMIT) ? 3 : JN_HJ_MINB)
+template <typename K, int MODE, int PU = (MODE == MODE_EMIT ? HJ_PU : 1)>
+__global__ void __launch_bounds__(HJ_T, JN_HJ_MINB)
 k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __restrict__ srows,
             const Item* __restrict__ items, const uint64_t* __restrict__ nitems_p, int bits,
-            unsigned long long* __restrict__ item_val,
-            unsigned long long* __restrict__ chk, const uint64_t* __restrict__ item_off,
-            jn_pair* __restrict__ out, unsigned int* __restrict__ err, uint64_t item_lo = 0,
-            uint64_t item_hi = ~0ull) {
+            unsigned long long* __restrict__ item_val, const uint64_t* __restrict__ item_off,
+            jn_pair* __restrict__ out, unsigned int* __restrict__ err) {
     using R = Row<K, false>;
-    using L = JoinSmem<K, MODE, CAP>;
+    using L = JoinSmem<K, MODE>;
     constexpr int TS = L::TS;
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* g_r = smem;
@@ -207,18 +202,15 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     // count-mode table
     K* o_key = reinterpret_cast<K*>(tab);
     uint32_t* o_cnt = reinterpret_cast<uint32_t*>(o_key + TS);
-    unsigned long long* o_f = reinterpret_cast<unsigned long long*>(o_cnt + TS);
     __shared__ unsigned long long tmp64[33];
     __shared__ uint32_t tmp32[33];
     __shared__ uint32_t s_cursor, s_mincnt;
-    __shared__ unsigned long long s_minf;
     __shared__ __align__(8) uint64_t bar_r, bar_s[2];
     const K KMIN = key_sentinel<K>();
 
     const int lane = threadIdx.x & 31;
-    // items [item_lo, min(*nitems_p, item_hi)) of the queue
-    const uint64_t nitems = min(*nitems_p, item_hi);
-    uint64_t it = item_lo + blockIdx.x;
+    const uint64_t nitems = *nitems_p;
+    uint64_t it = blockIdx.x;
     if (it >= nitems) return;
     Item d = items[it];
     // S-chunk stream: chunk q of this block sits in buffer q & 1; thread 0
@@ -269,9 +261,8 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         // slots this item uses: four times its R rows (at most the table) -- a
         // slot is picked by multiply-shift, so any count works.  At a load of
         // a quarter, a lookup that misses (most of them in a selective join)
-        // scans about 1.4 slots; at a half, 2.5.  The skewed variant keeps the
-        // whole table
-        const int ts = (MERGE || MODE == MODE_EMIT) ? TS : min(TS, max(64, 4 * rn));
+        // scans about 1.4 slots; at a half, 2.5
+        const int ts = MODE == MODE_EMIT ? TS : min(TS, max(64, 4 * rn));
         if (MODE == MODE_EMIT) {
             for (int i = threadIdx.x; i <= TS; i += HJ_T) {
                 e_tab[i].key = KMIN;
@@ -281,12 +272,8 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
             for (int i = threadIdx.x; i < ts; i += HJ_T) {
                 o_key[i] = KMIN;
                 o_cnt[i] = 0;
-                if (MODE == MODE_AGG) o_f[i] = 0;
             }
-            if (threadIdx.x == 0) {
-                s_mincnt = 0;
-                s_minf = 0;
-            }
+            if (threadIdx.x == 0) s_mincnt = 0;
         }
         if (__syncthreads_or(!mbar_wait(&bar_r, pr, err))) {
             failed = true;
@@ -297,23 +284,8 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         const R* rrow = reinterpret_cast<const R*>(g_r + span_off<R>(d.rbeg));
         if (MODE == MODE_EMIT) {
             // ---- build: one slot per distinct key, then its payloads as one run ----
-            // MERGE (skewed input): lanes of a warp holding the same key update
-            // their slot once, to spare contended shared atomics
-            const int rnw = MERGE ? (rn + 31) & ~31 : rn;
-            for (int i = threadIdx.x; i < rnw; i += HJ_T) {
-                const bool in = i < rn;
-                R x;
-                x.key = KMIN;
-                x.pay = 0;
-                if (in) x = rrow[i];
-                uint32_t cnt = 1;
-                if (MERGE) {
-                    const unsigned act = __ballot_sync(0xffffffffu, in);
-                    if (!in) continue;
-                    const unsigned peers = __match_any_sync(act, x.key);
-                    if (lane != __ffs(peers) - 1) continue;
-                    cnt = __popc(peers);
-                }
+            for (int i = threadIdx.x; i < rn; i += HJ_T) {
+                const R x = rrow[i];
                 uint32_t h = TS;  // the sentinel key keeps its own slot
                 if (x.key != KMIN) {
                     h = oa_slot(khash(x.key), bits, TS);
@@ -328,7 +300,7 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
                         h = (h + 1 == (uint32_t)TS) ? 0u : h + 1;
                     }
                 }
-                atomicAdd(&e_tab[h].packed, cnt << 16);
+                atomicAdd(&e_tab[h].packed, 1u << 16);
             }
             __syncthreads();
             // run starts: exclusive scan of the slot counts into the low halves
@@ -350,64 +322,23 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
             }
             __syncthreads();
             // payloads into their runs; each cursor ends at its run's end
-            for (int i = threadIdx.x; i < rnw; i += HJ_T) {
-                const bool in = i < rn;
-                R x;
-                x.key = KMIN;
-                x.pay = 0;
-                if (in) x = rrow[i];
+            for (int i = threadIdx.x; i < rn; i += HJ_T) {
+                const R x = rrow[i];
                 uint32_t h = TS;
-                if (in && x.key != KMIN) {
+                if (x.key != KMIN) {
                     h = oa_slot(khash(x.key), bits, TS);
                     for (int probe = 0; probe < TS && e_tab[h].key != x.key; probe++)
                         h = (h + 1 == (uint32_t)TS) ? 0u : h + 1;
                 }
-                uint32_t pos;
-                if (MERGE) {
-                    const unsigned act = __ballot_sync(0xffffffffu, in);
-                    if (!in) continue;
-                    const unsigned peers = __match_any_sync(act, x.key);
-                    const int leader = __ffs(peers) - 1;
-                    uint32_t b0 = 0;
-                    if (lane == leader) b0 = atomicAdd(&e_tab[h].packed, (uint32_t)__popc(peers));
-                    b0 = __shfl_sync(peers, b0, leader);
-                    pos = (b0 & 0xffffu) + __popc(peers & ((1u << lane) - 1));
-                } else {
-                    if (!in) continue;
-                    pos = atomicAdd(&e_tab[h].packed, 1u) & 0xffffu;
-                }
+                const uint32_t pos = atomicAdd(&e_tab[h].packed, 1u) & 0xffffu;
                 s_pay[pos] = x.pay;
             }
         } else {
-            // ---- build: fold equal keys into one slot (key, count [, sum f]) ----
-            // MERGE (skewed input): lanes of a warp holding the same key insert
-            // once, with their count, to spare contended shared atomics
-            const int rnw = MERGE ? (rn + 31) & ~31 : rn;
-            for (int i = threadIdx.x; i < rnw; i += HJ_T) {
-                const bool in = i < rn;
-                R x;
-                x.key = KMIN;
-                x.pay = 0;
-                if (in) x = rrow[i];
-                uint32_t cnt = 1;
-                unsigned long long fv = 0;
-                if (MERGE) {
-                    const unsigned act = __ballot_sync(0xffffffffu, in);
-                    if (!in) continue;
-                    const unsigned peers = __match_any_sync(act, x.key);
-                    if (MODE == MODE_AGG) {
-                        // sum f over the peer group, gathered by its leader
-                        const unsigned long long mine = chk_f(x.pay);
-                        for (unsigned m = peers; m; m &= m - 1) fv += __shfl_sync(peers, mine, __ffs(m) - 1);
-                    }
-                    if ((threadIdx.x & 31) != (unsigned)(__ffs(peers) - 1)) continue;
-                    cnt = __popc(peers);
-                } else if (MODE == MODE_AGG) {
-                    fv = chk_f(x.pay);
-                }
+            // ---- build: fold equal keys into one slot (key, count) ----
+            for (int i = threadIdx.x; i < rn; i += HJ_T) {
+                const R x = rrow[i];
                 if (x.key == KMIN) {  // the empty-slot marker itself: kept aside
-                    atomicAdd(&s_mincnt, cnt);
-                    if (MODE == MODE_AGG) atomicAdd(&s_minf, fv);
+                    atomicAdd(&s_mincnt, 1u);
                     continue;
                 }
                 uint32_t h = oa_slot(khash(x.key), bits, ts);
@@ -419,8 +350,7 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
                         old = (K)atomicCAS(reinterpret_cast<unsigned long long*>(o_key) + h,
                                            (unsigned long long)KMIN, (unsigned long long)x.key);
                     if (old == KMIN || old == x.key) {
-                        atomicAdd(&o_cnt[h], cnt);
-                        if (MODE == MODE_AGG) atomicAdd(&o_f[h], fv);
+                        atomicAdd(&o_cnt[h], 1u);
                         break;
                     }
                     h = (h + 1 == (uint32_t)ts) ? 0u : h + 1;
@@ -432,7 +362,7 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         if (threadIdx.x == 0 && has_next) stage_span<R>(rrows, dn.rbeg, dn.rn, g_r, &bar_r);
         r_pending = has_next;
         // ---- probe with every S chunk of the partition ----
-        unsigned long long acc = 0, csum = 0;
+        unsigned long long acc = 0;
         const uint64_t ibase = MODE == MODE_EMIT ? item_off[it] : 0;
         const int nsc = (d.sn + HJ_SCH - 1) / HJ_SCH;
         for (int sc = 0; sc < nsc; sc++) {
@@ -451,7 +381,6 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
             for (int r = 0; r < rounds; r += PU) {
                 R x[PU];
                 uint32_t m[PU], beg[PU];
-                unsigned long long fs[PU];
 #pragma unroll
                 for (int u = 0; u < PU; u++) {
                     const int j = (r + u) * HJ_T + threadIdx.x;
@@ -459,7 +388,6 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
                     x[u].pay = 0;
                     m[u] = 0;
                     beg[u] = 0;
-                    fs[u] = 0;
                     if (j < sn) x[u] = srow[j];
                 }
 #pragma unroll
@@ -486,14 +414,12 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
                         beg[u] = (p & 0xffffu) - m[u];
                     } else if (x[u].key == KMIN) {
                         m[u] = s_mincnt;
-                        if (MODE == MODE_AGG) fs[u] = s_minf;
                     } else {
                         uint32_t h = oa_slot(khash(x[u].key), bits, ts);
                         for (int probe = 0; probe < ts; probe++) {
                             const K kk = o_key[h];
                             if (kk == x[u].key) {
                                 m[u] = o_cnt[h];
-                                if (MODE == MODE_AGG) fs[u] = o_f[h];
                                 break;
                             }
                             if (kk == KMIN) break;
@@ -533,10 +459,7 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
                     }
                 } else {
 #pragma unroll
-                    for (int u = 0; u < PU; u++) {
-                        acc += m[u];
-                        if (MODE == MODE_AGG && m[u]) csum += fs[u] * chk_g(x[u].pay);
-                    }
+                    for (int u = 0; u < PU; u++) acc += m[u];
                 }
             }
             __syncthreads();  // this S buffer is free: stage the chunk after next
@@ -546,10 +469,6 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         if (failed) break;
         if (MODE != MODE_EMIT) {
             const unsigned long long tot = block_sum(acc, tmp64);
-            if (MODE == MODE_AGG) {
-                const unsigned long long ct = block_sum(csum, tmp64);
-                if (threadIdx.x == 0 && ct) atomicAdd(chk, ct);
-            }
             if (threadIdx.x == 0) item_val[it] = tot;
         }
         if (!has_next) break;
@@ -566,22 +485,6 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         if (r_pending) mbar_wait(&bar_r, pr, nullptr);
         for (uint32_t q = qc; q < s_qp; q++) mbar_wait(&bar_s[q & 1], (q >> 1) & 1, nullptr);
     }
-}
-
-template <typename K>
-static size_t hash_smem(int mode, int cap = cap_of<K>()) {
-    constexpr int C = cap_of<K>(), H = C / 2;
-    if (mode == MODE_EMIT) return cap == C ? JoinSmem<K, MODE_EMIT>::BYTES : JoinSmem<K, MODE_EMIT, H>::BYTES;
-    if (mode == MODE_AGG) return cap == C ? JoinSmem<K, MODE_AGG>::BYTES : JoinSmem<K, MODE_AGG, H>::BYTES;
-    return cap == C ? JoinSmem<K, MODE_COUNT>::BYTES : JoinSmem<K, MODE_COUNT, H>::BYTES;
-}
-
-// The skewed-input join kernel for a table of `cap` R rows (the full table or
-// half of it).
-template <typename K, int MODE>
-static auto hash_join_kernel(int cap) {
-    constexpr int C = cap_of<K>(), H = C / 2;
-    return cap == C ? k_hash_join<K, MODE, true, C> : k_hash_join<K, MODE, true, H>;
 }
 
 static int persistent_grid(jn_ctx* c, const void* fn, int threads, size_t smem) {
@@ -606,6 +509,7 @@ struct Partitioned {
     uint32_t* pcnt = nullptr;
     Row<K, false>* hrows = nullptr; // heavy rows grouped by heavy key
     uint64_t* hoff = nullptr;       // HV_MAX + 1 offsets
+    const uint64_t* hseg = nullptr; // or, ungrouped, the two bounds of the heavy rows in hrows
     PartView view() const { return off ? PartView{off, nullptr, nullptr} : PartView{nullptr, pbeg, pcnt}; }
 };
 
@@ -742,11 +646,12 @@ static jn_status group_heavy(jn_ctx* c, Scratch& s, const Row<K, false>* rows, u
 // the key hash, plus the heavy digit F1), then one block per region splits it
 // into 2^b2 partitions of rows.  With `filter`, table `first` builds the
 // key-presence slices and the other table is thinned by them (Algorithm 1's
-// pre-filter, one side).  d_small[0] / [1] receive R's / S's rows kept.
+// pre-filter, one side).  Heavy rows are grouped by key with `group` (to write
+// their pairs), else left where level 1 put them.  d_small[0] / [1] receive R's / S's rows kept.
 template <typename K, typename D1>
 static jn_status region_partition(jn_ctx* c, Scratch& s, const Cols<K>& R, const Cols<K>& S, int b1, int b2, D1 d1,
-                                  const HeavySet<K>* hs, bool filter, int first, int fb, Partitioned<K>* PR,
-                                  Partitioned<K>* PS, uint64_t* d_small) {
+                                  const HeavySet<K>* hs, bool group, bool filter, int first, int fb,
+                                  Partitioned<K>* PR, Partitioned<K>* PS, uint64_t* d_small) {
     using RW = Row<K, false>;
     using SH = RgShape<K>;
     const int F1 = 1 << b1, F2 = 1 << b2;
@@ -808,7 +713,12 @@ static jn_status region_partition(jn_ctx* c, Scratch& s, const Cols<K>& R, const
         P[t]->rows = rows;
         P[t]->pbeg = pb;
         P[t]->pcnt = pc;
-        if (hs) JN_TRY(group_heavy<K>(c, s, (const RW*)rows1[t], (uint64_t)n + HJ_PAD, start1[t] + F1, *hs, P[t]));
+        if (hs && group) {
+            JN_TRY(group_heavy<K>(c, s, (const RW*)rows1[t], (uint64_t)n + HJ_PAD, start1[t] + F1, *hs, P[t]));
+        } else if (hs) {
+            P[t]->hrows = rows1[t];
+            P[t]->hseg = start1[t] + F1;
+        }
     }
     return JN_OK;
 }
@@ -1002,7 +912,7 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
         return JN_OK;
     };
     auto region_all = [&](auto d1) -> jn_status {
-        return region_partition<K, decltype(d1)>(c, s, R, S, b1, b2, d1, heavy ? &hs : nullptr, fside != 0,
+        return region_partition<K, decltype(d1)>(c, s, R, S, b1, b2, d1, heavy ? &hs : nullptr, mode == MODE_EMIT, fside != 0,
                                                  (fside & 1) ? 0 : 1, fb, &PR, &PS, d_small);
     };
     if (heavy) {
@@ -1030,10 +940,7 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     uint64_t h[16];
     JN_TRY(launch(c, K_MISC, k_copy_words, dim3(1), dim3(32), 0, (const uint64_t*)(iprefix + P),
                   d_small + 2, 1));
-    if (heavy) JN_CUDA(c, cudaMemcpyAsync(d_small + 7, d_hcount, 4, cudaMemcpyDeviceToDevice, c->stream));
     JN_TRY(read_back(c, d_small, h, 16));
-    // many frequent keys in the sample: expect duplicate-heavy partitions too
-    const bool skewed = heavy && (h[7] & 0xffffffffu) >= 64;
     const uint64_t nitems = h[2];
     info.r_survivors = h[0];
     info.s_survivors = h[1];
@@ -1054,11 +961,10 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     uint64_t* ioff = nullptr;
     JN_TRY(s.get(&idesc, nitems + 1));
     RW* rsorted = nullptr;  // sort-merge: the R chunks sorted by key
-    // once: the hash join of an input without many frequent keys finds its
-    // pairs and keeps them in one pass (jn_partjoin.cuh); the others count per
-    // item, scan, and join again to write
-    const bool once = !sort_merge && !skewed;
-    const int jcap = cap == cap_of<K>() / 2 ? cap : cap_of<K>();  // k_hash_join comes in two sizes
+    // once: the hash join finds its pairs and keeps them in one pass
+    // (jn_partjoin.cuh); the sort-merge join counts per item, scans, and joins
+    // again to write
+    const bool once = !sort_merge;
     DirectSmall* small = nullptr;
     jn_pair* staged = nullptr;
     uint32_t segs = 1;
@@ -1116,22 +1022,28 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             JN_TRY(launch(c, K_SORT_COUNT, kc, dim3(gj), dim3(SJ_T), smc, (const RW*)rsorted, (const RW*)PS.rows,
                           (const Item*)idesc, (const uint64_t*)(iprefix + P), cap, ival, chk,
                           (const uint64_t*)nullptr, (jn_pair*)nullptr, (uint64_t)0, ~0ull));
-        } else if (once) {
-            JN_TRY(join_once(room ? MODE_EMIT : cm, staged, segs, room));
         } else {
-            const size_t smc = hash_smem<K>(cm, jcap);
-            auto kc = cm == MODE_AGG ? hash_join_kernel<K, MODE_AGG>(jcap)
-                                     : hash_join_kernel<K, MODE_COUNT>(jcap);
-            const int gj = (int)min((uint64_t)persistent_grid(c, (const void*)kc, HJ_T, smc), nitems);
-            JN_TRY(launch(c, K_HASH_COUNT, kc, dim3(gj), dim3(HJ_T), smc, (const RW*)PR.rows, (const RW*)PS.rows,
-                          (const Item*)idesc, (const uint64_t*)(iprefix + P), b, ival, chk,
-                          (const uint64_t*)nullptr, (jn_pair*)nullptr, c->d_err, (uint64_t)0, ~0ull));
+            JN_TRY(join_once(room ? MODE_EMIT : cm, staged, segs, room));
         }
     }
     if (!once) JN_TRY(scan_u64(c, reinterpret_cast<const uint64_t*>(ival), ioff, (int64_t)nitems));
     // ---- heavy keys: c_R(h) * c_S(h) pairs each ----
     uint64_t *hp = nullptr, *hpoff = nullptr, *hch = nullptr, *hchp = nullptr;
-    if (heavy) {
+    if (heavy && PR.hseg) {
+        // counted or checksummed: rows and sums per heavy key
+        unsigned long long* hv;
+        JN_TRY(s.get(&hv, 4 * (size_t)HV_MAX));
+        JN_TRY(zero(c, hv, 8 * 4 * (size_t)HV_MAX));
+        const Partitioned<K>* part[2] = {&PR, &PS};
+        for (int t = 0; t < 2; t++)
+            JN_TRY(launch(c, K_HEAVY_SELECT, k_heavy_sums<K>, dim3(4 * c->num_sms), dim3(512), 0,
+                          (const RW*)part[t]->hrows, part[t]->hseg, hs, t, mode == MODE_AGG ? 1 : 0, hv + t * HV_MAX,
+                          hv + (2 + t) * HV_MAX));
+        JN_TRY(launch(c, K_HEAVY_SELECT, k_heavy_totals, dim3(1), dim3(1024), 0, (const unsigned long long*)hv,
+                      (const unsigned long long*)(hv + HV_MAX), (const unsigned long long*)(hv + 2 * HV_MAX),
+                      (const unsigned long long*)(hv + 3 * HV_MAX), d_small + 5, chk));
+        JN_CUDA(c, cudaMemcpyAsync(d_small + 6, d_hcount, 4, cudaMemcpyDeviceToDevice, c->stream));
+    } else if (heavy) {
         JN_TRY(s.get(&hp, HV_MAX));
         JN_TRY(s.get(&hpoff, HV_MAX + 1));
         JN_TRY(s.get(&hch, HV_MAX));
@@ -1211,24 +1123,16 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             JN_TRY(join_once(MODE_EMIT, plan->dev, 1, normal));
         }
     } else if (normal > 0) {
-        auto ke = hash_join_kernel<K, MODE_EMIT>(jcap);
         auto kse = k_sort_join<K, MODE_EMIT>;
-        const size_t sme = sort_merge ? SortJoinSmem<K>::bytes(cap, MODE_EMIT) : hash_smem<K>(MODE_EMIT, jcap);
-        const uint64_t pg = sort_merge ? (uint64_t)persistent_grid(c, (const void*)kse, SJ_T, sme)
-                                       : (uint64_t)persistent_grid(c, (const void*)ke, HJ_T, sme);
+        const size_t sme = SortJoinSmem<K>::bytes(cap, MODE_EMIT);
+        const uint64_t pg = (uint64_t)persistent_grid(c, (const void*)kse, SJ_T, sme);
         for (int k = 0; k < nsl; k++) {
             if (ib[k + 1] == ib[k]) continue;
             const int ge = (int)min(pg, ib[k + 1] - ib[k]);
-            if (sort_merge)
-                JN_TRY(launch(c, K_SORT_EMIT, kse, dim3(ge), dim3(SJ_T), sme, (const RW*)rsorted,
-                              (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P), cap,
-                              (unsigned long long*)nullptr, (unsigned long long*)nullptr, (const uint64_t*)ioff,
-                              plan->dev, ib[k], ib[k + 1]));
-            else
-                JN_TRY(launch(c, K_HASH_EMIT, ke, dim3(ge), dim3(HJ_T), sme, (const RW*)PR.rows,
-                              (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P), b,
-                              (unsigned long long*)nullptr, (unsigned long long*)nullptr, (const uint64_t*)ioff,
-                              plan->dev, c->d_err, ib[k], ib[k + 1]));
+            JN_TRY(launch(c, K_SORT_EMIT, kse, dim3(ge), dim3(SJ_T), sme, (const RW*)rsorted,
+                          (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P), cap,
+                          (unsigned long long*)nullptr, (unsigned long long*)nullptr, (const uint64_t*)ioff,
+                          plan->dev, ib[k], ib[k + 1]));
             if (nsl > 1) JN_TRY(copy_back(ob[k], ob[k + 1]));
         }
     }
@@ -1326,7 +1230,7 @@ struct HashBatchRun : BatchRun {
         int* d_bits;
         TileRef* d_tiles;
         uint64_t *d_ntiles, *start, *items, *d_off;
-        unsigned long long *hist, *cur, *ival, *chk;
+        unsigned long long *hist, *cur, *ival;
         JN_TRY(s->get(&d_segs, 2 * (size_t)n));
         JN_TRY(s->get(&d_bits, 2 * (size_t)n));
         JN_TRY(s->get(&d_tiles, ntiles + 1));
@@ -1340,7 +1244,6 @@ struct HashBatchRun : BatchRun {
         JN_TRY(s->get(&idesc, item_bound));
         JN_TRY(s->get(&ival, item_bound));
         JN_TRY(s->get(&ioff, item_bound + 1));
-        JN_TRY(s->get(&chk, 1));
         JN_TRY(s->get(&d_off, (size_t)n + 1));
         JN_CUDA(c, cudaMemcpyAsync(d_segs, segs.data(), sizeof(SegCols<K>) * segs.size(), cudaMemcpyHostToDevice,
                                    c->stream));
@@ -1358,7 +1261,6 @@ struct HashBatchRun : BatchRun {
         do {
             SegHashDigit dg{d_bits, 0};
             if ((st = zero(c, hist, sizeof(unsigned long long) * 2 * P)) != JN_OK) break;
-            if ((st = zero(c, chk, 8)) != JN_OK) break;
             if ((st = zero(c, ival, sizeof(unsigned long long) * item_bound)) != JN_OK) break;
             if ((st = launch(c, K_HIST, k_batch_hist<K>, dim3(4 * c->num_sms), dim3(SC_T), 0,
                              (const SegCols<K>*)d_segs, (const TileRef*)d_tiles, (const uint64_t*)d_ntiles, dg,
@@ -1386,12 +1288,12 @@ struct HashBatchRun : BatchRun {
                              PartView{roff, nullptr, nullptr}, PartView{soff, nullptr, nullptr},
                              (const uint64_t*)iprefix, (int)P, cap, idesc)) != JN_OK)
                 break;
-            auto kc = k_hash_join<K, MODE_COUNT, false>;
-            const size_t smc = hash_smem<K>(MODE_COUNT);
+            auto kc = k_hash_join<K, MODE_COUNT>;
+            const size_t smc = JoinSmem<K, MODE_COUNT>::BYTES;
             if ((st = launch(c, K_HASH_COUNT, kc, dim3(persistent_grid(c, (const void*)kc, HJ_T, smc)), dim3(HJ_T),
                              smc, (const RW*)prow, (const RW*)prow, (const Item*)idesc,
-                             (const uint64_t*)(iprefix + P), 10, ival, chk, (const uint64_t*)nullptr,
-                             (jn_pair*)nullptr, c->d_err, (uint64_t)0, ~0ull)) != JN_OK)
+                             (const uint64_t*)(iprefix + P), 10, ival, (const uint64_t*)nullptr, (jn_pair*)nullptr,
+                             c->d_err)) != JN_OK)
                 break;
             // items past the real count keep zero counts: scan the whole bound
             if ((st = scan_u64(c, reinterpret_cast<const uint64_t*>(ival), ioff, (int64_t)item_bound)) != JN_OK) break;
@@ -1418,11 +1320,10 @@ struct HashBatchRun : BatchRun {
         GraphPhase gp(c, c->tune.graphs != 0 && !c->profiling);
         JN_TRY(gp.begin());
         auto ke = k_hash_join<K, MODE_EMIT>;
-        const size_t sme = hash_smem<K>(MODE_EMIT);
+        const size_t sme = JoinSmem<K, MODE_EMIT>::BYTES;
         jn_status st = launch(c, K_HASH_EMIT, ke, dim3(persistent_grid(c, (const void*)ke, HJ_T, sme)), dim3(HJ_T),
                               sme, (const RW*)prow, (const RW*)prow, (const Item*)idesc, (const uint64_t*)(iprefix + P),
-                              10, (unsigned long long*)nullptr, (unsigned long long*)nullptr, (const uint64_t*)ioff,
-                              out, c->d_err, (uint64_t)0, ~0ull);
+                              10, (unsigned long long*)nullptr, (const uint64_t*)ioff, out, c->d_err);
         if (st != JN_OK) {
             gp.abort();
             return st;
