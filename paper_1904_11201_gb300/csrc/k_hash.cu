@@ -50,14 +50,11 @@ constexpr int HJ_SCH = JN_HJ_SCH;    // S rows per staged chunk
 #endif
 constexpr int HJ_PU = JN_HJ_PU;      // S rows a thread probes per round in the emit pass
 
-#ifndef JN_SLICE_PAIRS
-#define JN_SLICE_PAIRS (1ull << 24)  // host outputs of at least this many pairs are copied back in slices
-#endif
 constexpr int HJ_PAD = 16;         // rows of slack for 16-byte widened copies
-// the sort-merge kernels hold a chunk as 8 words per thread, index its rows in
-// 15 bits and sort it as a power-of-two network of at least 256 rows, in shared
-// memory sized for the chunk itself (int64 chunks are HJ_CAP / 2 rows)
-static_assert(HJ_CAP <= 8 * SJ_T && HJ_CAP < 0x8000, "R chunk larger than the sort-merge kernels hold");
+// the sort-merge kernels hold a chunk as 8 words per thread and sort it as a
+// power-of-two network of at least 256 rows, in shared memory sized for the
+// chunk itself (int64 chunks are HJ_CAP / 2 rows)
+static_assert(HJ_CAP <= SJ_CHUNK, "R chunk larger than the sort-merge kernels hold");
 static_assert((HJ_CAP & (HJ_CAP - 1)) == 0 && HJ_CAP >= 512,
               "R chunk must be a power of two of at least 512 rows (the sort network's size)");
 constexpr uint64_t CE_PAIRS = 1u << 16;  // cross-product pairs per work chunk
@@ -957,42 +954,41 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     if ((((uintptr_t)PR.rows) | ((uintptr_t)PS.rows)) & 15)
         return fail(c, JN_ERR_CUDA, "partition scratch is not 16-byte aligned");
     Item* idesc;
-    unsigned long long *ival = nullptr, *chk;
-    uint64_t* ioff = nullptr;
     JN_TRY(s.get(&idesc, nitems + 1));
     RW* rsorted = nullptr;  // sort-merge: the R chunks sorted by key
-    // once: the hash join finds its pairs and keeps them in one pass
-    // (jn_partjoin.cuh); the sort-merge join counts per item, scans, and joins
-    // again to write
-    const bool once = !sort_merge;
-    DirectSmall* small = nullptr;
+    // both joins find their pairs and keep them in one pass (jn_partjoin.cuh,
+    // jn_sortjoin.cuh)
+    DirectSmall* small;
     jn_pair* staged = nullptr;
     uint32_t segs = 1;
     uint64_t room = 0;  // pairs per segment
     Scratch ss(c);
-    if (once) {
-        JN_TRY(s.get(&small, 1));
-        JN_TRY(zero(c, small, sizeof(DirectSmall)));
-        chk = &small->lines[0].chk;
-        if (mode == MODE_EMIT && nitems && !c->mem_limit && !c->admit) {
-            // random keys on both sides match a surviving row 1.6 times; not
-            // under a limit that counts scratch
-            const uint64_t rows = max(h[0], h[1]);
-            segs = rows >= (1u << 23) ? DJ_SEGS : 1;
-            room = (rows + rows / 4 * 3) / segs + 4096;
-            if (ss.get(&staged, segs * room) != JN_OK) {
-                c->err.clear();
-                segs = 1;
-                room = 0;
-            }
+    JN_TRY(s.get(&small, 1));
+    JN_TRY(zero(c, small, sizeof(DirectSmall)));
+    unsigned long long* const chk = &small->lines[0].chk;
+    if (mode == MODE_EMIT && nitems && !c->mem_limit && !c->admit) {
+        // random keys on both sides match a surviving row 1.6 times; not
+        // under a limit that counts scratch
+        const uint64_t rows = max(h[0], h[1]);
+        segs = rows >= (1u << 23) ? DJ_SEGS : 1;
+        room = (rows + rows / 4 * 3) / segs + 4096;
+        if (ss.get(&staged, segs * room) != JN_OK) {
+            c->err.clear();
+            segs = 1;
+            room = 0;
         }
-    } else {
-        JN_TRY(s.get(&ival, nitems + 1));
-        JN_TRY(s.get(&ioff, nitems + 1));
-        JN_TRY(s.get(&chk, 1));
-        JN_TRY(zero(c, chk, 8));
     }
     auto join_once = [&](int m, jn_pair* to, uint32_t parts, uint64_t most) -> jn_status {
+        if (sort_merge) {
+            auto ks = m == MODE_EMIT ? k_sort_join<K, MODE_EMIT>
+                      : m == MODE_AGG ? k_sort_join<K, MODE_AGG>
+                                      : k_sort_join<K, MODE_COUNT>;
+            const size_t sm = SortJoinSmem<K>::bytes(cap, m);
+            const int g = (int)min((uint64_t)persistent_grid(c, (const void*)ks, SJ_T, sm), nitems);
+            return launch(c, m == MODE_EMIT ? K_SORT_EMIT : K_SORT_COUNT, ks, dim3(g), dim3(SJ_T), sm,
+                          (const RW*)rsorted, (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P),
+                          cap, b, small, to, parts, (unsigned long long)most);
+        }
         auto kj = m == MODE_EMIT ? k_part_join<K, MODE_EMIT>
                   : m == MODE_AGG ? k_part_join<K, MODE_AGG>
                                   : k_part_join<K, MODE_COUNT>;
@@ -1011,22 +1007,18 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
         if (sort_merge) {
             // every R chunk sorted by key once, into a copy the count and emit passes read
             JN_TRY(s.get(&rsorted, (size_t)R.n + HJ_PAD));
-            auto kso = k_sort_chunks<K>;
-            const size_t sms = SortJoinSmem<K>::sort_bytes(cap);
-            const int gs = (int)min((uint64_t)persistent_grid(c, (const void*)kso, SJ_T, sms), nitems);
-            JN_TRY(launch(c, K_SORT_CHUNKS, kso, dim3(gs), dim3(SJ_T), sms, (const RW*)PR.rows, rsorted,
-                          (const Item*)idesc, (const uint64_t*)(iprefix + P), cap));
-            auto kc = cm == MODE_AGG ? k_sort_join<K, MODE_AGG> : k_sort_join<K, MODE_COUNT>;
-            const size_t smc = SortJoinSmem<K>::bytes(cap, cm);
-            const int gj = (int)min((uint64_t)persistent_grid(c, (const void*)kc, SJ_T, smc), nitems);
-            JN_TRY(launch(c, K_SORT_COUNT, kc, dim3(gj), dim3(SJ_T), smc, (const RW*)rsorted, (const RW*)PS.rows,
-                          (const Item*)idesc, (const uint64_t*)(iprefix + P), cap, ival, chk,
-                          (const uint64_t*)nullptr, (jn_pair*)nullptr, (uint64_t)0, ~0ull));
-        } else {
-            JN_TRY(join_once(room ? MODE_EMIT : cm, staged, segs, room));
+            auto sort = [&](auto kso, bool narrow) -> jn_status {
+                const size_t sms = SortJoinSmem<K>::sort_bytes(cap, narrow);
+                const int gs = (int)min((uint64_t)persistent_grid(c, (const void*)kso, SJ_T, sms), nitems);
+                return launch(c, K_SORT_CHUNKS, kso, dim3(gs), dim3(SJ_T), sms, (const RW*)PR.rows, rsorted,
+                              (const Item*)idesc, (const uint64_t*)(iprefix + P), cap, b);
+            };
+            if constexpr (sizeof(K) == 8) JN_TRY(sort(k_sort_chunks<K>, false));
+            else if (b >= SJ_IDX) JN_TRY(sort(k_sort_chunks32<uint32_t>, true));
+            else JN_TRY(sort(k_sort_chunks32<uint64_t>, false));
         }
+        JN_TRY(join_once(room ? MODE_EMIT : cm, staged, segs, room));
     }
-    if (!once) JN_TRY(scan_u64(c, reinterpret_cast<const uint64_t*>(ival), ioff, (int64_t)nitems));
     // ---- heavy keys: c_R(h) * c_S(h) pairs each ----
     uint64_t *hp = nullptr, *hpoff = nullptr, *hch = nullptr, *hchp = nullptr;
     if (heavy && PR.hseg) {
@@ -1065,21 +1057,13 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
                       d_small + 5, 1));
         JN_CUDA(c, cudaMemcpyAsync(d_small + 6, d_hcount, 4, cudaMemcpyDeviceToDevice, c->stream));
     }
-    if (once) {
-        JN_TRY(direct_fetch(c, small, segs));
-    } else {
-        JN_TRY(launch(c, K_MISC, k_copy_words, dim3(1), dim3(32), 0, (const uint64_t*)(ioff + nitems),
-                      d_small + 3, 1));
-        JN_TRY(launch(c, K_MISC, k_copy_words, dim3(1), dim3(32), 0, (const uint64_t*)chk, d_small + 4, 1));
-    }
+    JN_TRY(direct_fetch(c, small, segs));
     uint64_t hc[4];
     JN_TRY(read_back(c, d_small + 3, hc, 4));
     DirectResult found;
-    if (once) {
-        direct_parse(c, segs, room, &found);
-        hc[0] = found.total;
-        hc[1] = found.chk;
-    }
+    direct_parse(c, segs, room, &found);
+    hc[0] = found.total;
+    hc[1] = found.chk;
     const uint64_t normal = hc[0], heavy_pairs = heavy ? hc[2] : 0;
     const uint64_t total = normal + heavy_pairs;
     res->count = total;
@@ -1092,48 +1076,13 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     // ---- 5. exact allocation and the emit pass ----
     if (!found.fits) ss.release();
     JN_TRY(out_prepare(c, s, total, *plan));
-    // A host output is copied back slice by slice (on the copy stream) while
-    // the later slices of the work queue emit: slice k's pairs are the
-    // contiguous range [ioff[ib[k]], ioff[ib[k + 1]]).
-    const int nsl = (!once && plan->host_copy && normal >= (uint64_t)JN_SLICE_PAIRS && nitems >= 64) ? 4 : 1;
-    uint64_t ib[5], ob[5] = {0, 0, 0, 0, 0};
-    for (int k = 0; k <= nsl; k++) ib[k] = nitems * (uint64_t)k / (uint64_t)nsl;
-    if (nsl > 1) {
-        for (int k = 0; k <= nsl; k++)
-            JN_CUDA(c, cudaMemcpyAsync(d_small + 8 + k, ioff + ib[k], 8, cudaMemcpyDeviceToDevice, c->stream));
-        JN_TRY(read_back(c, d_small + 8, ob, nsl + 1));
-        if (!c->copy_stream) JN_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
-    }
-    auto copy_back = [&](uint64_t lo, uint64_t hi) -> jn_status {  // pairs [lo, hi) to the caller's buffer
-        if (hi <= lo) return JN_OK;
-        cudaEvent_t e;
-        JN_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        cudaEventRecord(e, c->stream);
-        cudaStreamWaitEvent(c->copy_stream, e, 0);
-        cudaEventDestroy(e);
-        JN_CUDA(c, cudaMemcpyAsync(*plan->user_out + lo, plan->dev + lo, (hi - lo) * sizeof(jn_pair),
-                                   cudaMemcpyDefault, c->copy_stream));
-        return JN_OK;
-    };
-    if (once && normal > 0) {
+    if (normal > 0) {
         if (room && found.fits) {
-            JN_TRY((direct_gather<uint64_t, 1>(c, K_HASH_EMIT, staged, segs, room, found, plan->dev)));
+            JN_TRY((direct_gather<uint64_t, 1>(c, sort_merge ? K_SORT_EMIT : K_HASH_EMIT, staged, segs, room, found,
+                                               plan->dev)));
         } else {
             JN_TRY(zero(c, &small->lines[0].total, 8));
             JN_TRY(join_once(MODE_EMIT, plan->dev, 1, normal));
-        }
-    } else if (normal > 0) {
-        auto kse = k_sort_join<K, MODE_EMIT>;
-        const size_t sme = SortJoinSmem<K>::bytes(cap, MODE_EMIT);
-        const uint64_t pg = (uint64_t)persistent_grid(c, (const void*)kse, SJ_T, sme);
-        for (int k = 0; k < nsl; k++) {
-            if (ib[k + 1] == ib[k]) continue;
-            const int ge = (int)min(pg, ib[k + 1] - ib[k]);
-            JN_TRY(launch(c, K_SORT_EMIT, kse, dim3(ge), dim3(SJ_T), sme, (const RW*)rsorted,
-                          (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P), cap,
-                          (unsigned long long*)nullptr, (unsigned long long*)nullptr, (const uint64_t*)ioff,
-                          plan->dev, ib[k], ib[k + 1]));
-            if (nsl > 1) JN_TRY(copy_back(ob[k], ob[k + 1]));
         }
     }
     if (heavy_pairs > 0) {
@@ -1141,15 +1090,6 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
                       (const uint64_t*)PR.hoff, (const RW*)PS.hrows, (const uint64_t*)PS.hoff,
                       (const uint64_t*)hpoff, (const uint64_t*)hchp, HV_MAX, (uint64_t)CE_PAIRS, normal,
                       plan->dev));
-    }
-    if (nsl > 1) {
-        JN_TRY(copy_back(normal, total));
-        cudaEvent_t e;  // the run ends when its last copy has landed
-        JN_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        cudaEventRecord(e, c->copy_stream);
-        cudaStreamWaitEvent(c->stream, e, 0);
-        cudaEventDestroy(e);
-        plan->copied = true;
     }
     JN_TRY(out_finish(c, total, *plan));
     return JN_OK;
