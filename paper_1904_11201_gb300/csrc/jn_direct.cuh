@@ -522,6 +522,18 @@ struct DirectCounts {
     unsigned long long n[DJ_SEGS];
 };
 
+// Where a partition join's pairs go.  Work item i's pairs belong to segment
+// i % segs: its own part of scratch in the first pass or, once the segments'
+// pairs are counted, of the output.  A launch takes the segments [lo, lo + w);
+// its grid is a multiple of w, so a block stays with one segment.
+struct PairSegs {
+    uint32_t segs, lo, w;
+    unsigned long long at[DJ_SEGS], cap[DJ_SEGS];
+    __device__ __forceinline__ uint32_t seg() const { return lo + blockIdx.x % w; }
+    __device__ __forceinline__ uint64_t first() const { return (uint64_t)(blockIdx.x / w) * segs + seg(); }
+    __device__ __forceinline__ uint64_t step() const { return (uint64_t)(gridDim.x / w) * segs; }
+};
+
 // The segments of staged results, one after the other, into out.  PER words
 // of type T per result.
 template <typename T, int PER>

@@ -78,7 +78,7 @@ template <typename K, int MODE>
 __global__ void __launch_bounds__(PJ_T, MODE == MODE_EMIT ? JN_PJ_MINBE : JN_PJ_MINB)
 k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __restrict__ srows,
             const Item* __restrict__ items, const uint64_t* __restrict__ nitems_p, int cap_rows, int bits,
-            DirectSmall* __restrict__ small, jn_pair* __restrict__ out, uint32_t segs, unsigned long long cap,
+            DirectSmall* __restrict__ small, jn_pair* __restrict__ out, const __grid_constant__ PairSegs ps,
             unsigned int* __restrict__ err) {
     using R = Row<K, false>;
     using L = PartJoinSmem<K, MODE>;
@@ -95,7 +95,9 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     constexpr int PU = MODE == MODE_EMIT ? JN_PJ_PUE : JN_PJ_PU;  // S rows a thread loads at once
     const int tid = threadIdx.x, lane = tid & 31;
     const uint64_t nitems = *nitems_p;
-    const uint32_t seg = blockIdx.x % segs;
+    const uint32_t seg = ps.seg();
+    const uint64_t first_item = ps.first(), step = ps.step();
+    const unsigned long long cap = ps.cap[seg];
     if (tid == 0) {
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -103,7 +105,7 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     __syncthreads();
     // the warp's pairs on their way out
     int2* const buf = MODE == MODE_EMIT ? s_out + (tid >> 5) * 2 * PJ_BUF : nullptr;
-    int2* const gout = reinterpret_cast<int2*>(out) + seg * cap;
+    int2* const gout = reinterpret_cast<int2*>(out) + ps.at[seg];
     uint32_t fill = 0;
     auto reserve = [&](unsigned long long n, unsigned long long* at) {
         unsigned long long a = 0;
@@ -122,8 +124,8 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     unsigned long long acc = 0, csum = 0;
     uint32_t phase = 0;
     Item d{};
-    if (blockIdx.x < nitems) d = items[blockIdx.x];
-    for (uint64_t it = blockIdx.x; it < nitems; it += gridDim.x) {
+    if (first_item < nitems) d = items[first_item];
+    for (uint64_t it = first_item; it < nitems; it += step) {
         const int rn = d.rn, sn = d.sn;
         const uint64_t lo = (d.rbeg * sizeof(R)) & ~15ull;
         // bytes of rows [beg, beg + n), widened to 16-byte boundaries
@@ -137,8 +139,8 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         }
         // the next item's rows start on their way to L2
         Item dn{};
-        if (it + gridDim.x < nitems) {
-            dn = items[it + gridDim.x];
+        if (it + step < nitems) {
+            dn = items[it + step];
             if (tid == 0)
                 l2_prefetch(reinterpret_cast<const unsigned char*>(rrows) + ((dn.rbeg * sizeof(R)) & ~15ull),
                             span(dn.rbeg, dn.rn));
@@ -326,7 +328,7 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     acc = block_sum(acc, tmp64);
     if (MODE == MODE_AGG) csum = block_sum(csum, tmp64);
     if (tid == 0) {
-        if (acc) atomicAdd(&small->lines[0].total, acc);
+        if (acc) atomicAdd(&small->lines[seg].total, acc);
         if (MODE == MODE_AGG && csum) atomicAdd(&small->lines[0].chk, csum);
     }
 }

@@ -288,7 +288,7 @@ template <typename K, int MODE>
 __global__ void __launch_bounds__(SJ_T, JN_SJ_MINB)
 k_sort_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __restrict__ srows,
             const Item* __restrict__ items, const uint64_t* __restrict__ nitems_p, int cap_rows, int bits,
-            DirectSmall* __restrict__ small, jn_pair* __restrict__ out, uint32_t segs, unsigned long long cap) {
+            DirectSmall* __restrict__ small, jn_pair* __restrict__ out, const __grid_constant__ PairSegs ps) {
     using U = typename SortJoinSmem<K>::U;
     extern __shared__ __align__(128) unsigned char smem[];
     U* s_k = reinterpret_cast<U*>(smem);
@@ -300,10 +300,12 @@ k_sort_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     constexpr int PER = JN_SJ_PER;  // S rows a thread searches for at once
     const int tid = threadIdx.x, lane = tid & 31;
     const uint64_t nitems = *nitems_p;
-    const uint32_t seg = blockIdx.x % segs;
-    jn_pair* const gout = out + seg * cap;
+    const uint32_t seg = ps.seg();
+    const unsigned long long cap = ps.cap[seg];
+    jn_pair* const gout = out + ps.at[seg];
     unsigned long long acc = 0, csum = 0;
-    for (uint64_t it = blockIdx.x; it < nitems; it += gridDim.x) {
+    const uint64_t next = ps.step();
+    for (uint64_t it = ps.first(); it < nitems; it += next) {
         const Item d = items[it];
         const uint32_t rn = (uint32_t)d.rn;
         for (uint32_t i = tid; i < rn; i += SJ_T) {  // the chunk, sorted by key
@@ -417,7 +419,7 @@ k_sort_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     acc = block_sum(acc, tmp64);
     if (MODE == MODE_AGG) csum = block_sum(csum, tmp64);
     if (tid == 0) {
-        if (acc) atomicAdd(&small->lines[0].total, acc);
+        if (acc) atomicAdd(&small->lines[seg].total, acc);
         if (MODE == MODE_AGG && csum) atomicAdd(&small->lines[0].chk, csum);
     }
 }

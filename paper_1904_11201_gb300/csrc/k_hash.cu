@@ -960,34 +960,47 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     // jn_sortjoin.cuh)
     DirectSmall* small;
     jn_pair* staged = nullptr;
-    uint32_t segs = 1;
-    uint64_t room = 0;  // pairs per segment
+    const uint32_t segs = nitems >= 64 * DJ_SEGS ? DJ_SEGS : 1;  // cursors: PairSegs
+    uint64_t room = 0;                                           // pairs kept per segment
     Scratch ss(c);
     JN_TRY(s.get(&small, 1));
     JN_TRY(zero(c, small, sizeof(DirectSmall)));
     unsigned long long* const chk = &small->lines[0].chk;
-    if (mode == MODE_EMIT && nitems && !c->mem_limit && !c->admit) {
-        // random keys on both sides match a surviving row 1.6 times; not
-        // under a limit that counts scratch
-        const uint64_t rows = max(h[0], h[1]);
-        segs = rows >= (1u << 23) ? DJ_SEGS : 1;
+    const uint64_t rows = max(h[0], h[1]);
+    // a large result on its way to host memory is counted first and then
+    // copied there, two segments at a time, while the next are written: page-
+    // locked host buffers, n x n random int32 rows, ms (kept in scratch first):
+    // 2^24 1.61 (1.73), 2^26 5.15 (5.71), 2^28 19.6 (22.0)
+    const bool sliced = mode == MODE_EMIT && segs > 1 && rows >= (1u << 23) && plan->user_out && *plan->user_out &&
+                        !is_device_pointer(*plan->user_out);
+    if (mode == MODE_EMIT && nitems && !sliced && !c->admit) {
+        // random keys on both sides match a surviving row 1.6 times; under a
+        // limit that counts scratch only with place for as many bytes of output
+        // (2^28 x 2^28 random int32 rows: 10.7 ms, 11.3 counted first and then
+        // written)
         room = (rows + rows / 4 * 3) / segs + 4096;
-        if (ss.get(&staged, segs * room) != JN_OK) {
+        if (c->mem_limit && c->scratch_bytes + 2 * segs * room * sizeof(jn_pair) > c->mem_limit) {
+            room = 0;
+        } else if (ss.get(&staged, segs * room) != JN_OK) {
             c->err.clear();
-            segs = 1;
             room = 0;
         }
     }
-    auto join_once = [&](int m, jn_pair* to, uint32_t parts, uint64_t most) -> jn_status {
+    auto join_once = [&](int m, jn_pair* to, const PairSegs& ps) -> jn_status {
+        // as many blocks as are resident, a multiple of the launch's segments
+        auto grid = [&](uint64_t resident) {
+            const uint64_t g = min(resident, nitems);
+            return dim3((unsigned)max(g - g % ps.w, (uint64_t)ps.w));
+        };
         if (sort_merge) {
             auto ks = m == MODE_EMIT ? k_sort_join<K, MODE_EMIT>
                       : m == MODE_AGG ? k_sort_join<K, MODE_AGG>
                                       : k_sort_join<K, MODE_COUNT>;
             const size_t sm = SortJoinSmem<K>::bytes(cap, m);
-            const int g = (int)min((uint64_t)persistent_grid(c, (const void*)ks, SJ_T, sm), nitems);
-            return launch(c, m == MODE_EMIT ? K_SORT_EMIT : K_SORT_COUNT, ks, dim3(g), dim3(SJ_T), sm,
+            return launch(c, m == MODE_EMIT ? K_SORT_EMIT : K_SORT_COUNT, ks,
+                          grid((uint64_t)persistent_grid(c, (const void*)ks, SJ_T, sm)), dim3(SJ_T), sm,
                           (const RW*)rsorted, (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P),
-                          cap, b, small, to, parts, (unsigned long long)most);
+                          cap, b, small, to, ps);
         }
         auto kj = m == MODE_EMIT ? k_part_join<K, MODE_EMIT>
                   : m == MODE_AGG ? k_part_join<K, MODE_AGG>
@@ -995,11 +1008,17 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
         const size_t sm = m == MODE_EMIT ? PartJoinSmem<K, MODE_EMIT>::bytes(cap)
                           : m == MODE_AGG ? PartJoinSmem<K, MODE_AGG>::bytes(cap)
                                           : PartJoinSmem<K, MODE_COUNT>::bytes(cap);
-        const int g = (int)min((uint64_t)persistent_grid(c, (const void*)kj, PJ_T, sm), nitems);
-        return launch(c, m == MODE_EMIT ? K_HASH_EMIT : K_HASH_COUNT, kj, dim3(g), dim3(PJ_T), sm, (const RW*)PR.rows,
-                      (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P), cap, b, small, to, parts,
-                      (unsigned long long)most, c->d_err);
+        return launch(c, m == MODE_EMIT ? K_HASH_EMIT : K_HASH_COUNT, kj,
+                      grid((uint64_t)persistent_grid(c, (const void*)kj, PJ_T, sm)), dim3(PJ_T), sm, (const RW*)PR.rows,
+                      (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P), cap, b, small, to, ps,
+                      c->d_err);
     };
+    PairSegs ps{};
+    ps.segs = ps.w = segs;
+    for (uint32_t i = 0; i < segs; i++) {
+        ps.at[i] = i * room;
+        ps.cap[i] = room;
+    }
     if (nitems) {
         JN_TRY(launch(c, K_ITEMS, k_item_desc, dim3((unsigned)ceil_div(nitems, 256)), dim3(256), 0, PR.view(),
                       PS.view(), (const uint64_t*)iprefix, P, cap, idesc));
@@ -1017,7 +1036,7 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             else if (b >= SJ_IDX) JN_TRY(sort(k_sort_chunks32<uint32_t>, true));
             else JN_TRY(sort(k_sort_chunks32<uint64_t>, false));
         }
-        JN_TRY(join_once(room ? MODE_EMIT : cm, staged, segs, room));
+        JN_TRY(join_once(room ? MODE_EMIT : cm, staged, ps));
     }
     // ---- heavy keys: c_R(h) * c_S(h) pairs each ----
     uint64_t *hp = nullptr, *hpoff = nullptr, *hch = nullptr, *hchp = nullptr;
@@ -1074,15 +1093,50 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     info.cartesian_bound = h[15] + heavy_pairs;  // the frequent keys' cross products are exact
     if (mode != MODE_EMIT) return JN_OK;
     // ---- 5. exact allocation and the emit pass ----
-    if (!found.fits) ss.release();
+    // kept pairs that did not fit, or that a limit wants for the output
+    if (!found.fits || (c->mem_limit && c->scratch_bytes + total * sizeof(jn_pair) > c->mem_limit)) {
+        ss.release();
+        room = 0;
+    }
     JN_TRY(out_prepare(c, s, total, *plan));
+    uint64_t copied = 0;  // pairs that are on their way to the caller's buffer
     if (normal > 0) {
         if (room && found.fits) {
             JN_TRY((direct_gather<uint64_t, 1>(c, sort_merge ? K_SORT_EMIT : K_HASH_EMIT, staged, segs, room, found,
                                                plan->dev)));
         } else {
-            JN_TRY(zero(c, &small->lines[0].total, 8));
-            JN_TRY(join_once(MODE_EMIT, plan->dev, 1, normal));
+            // the segments' pairs are counted: each has its place in the output
+            JN_TRY(zero(c, small, sizeof(DirectSmall)));
+            unsigned long long at = 0;
+            for (uint32_t i = 0; i < segs; i++) {
+                ps.at[i] = at;
+                ps.cap[i] = found.counts.n[i];
+                at += ps.cap[i];
+            }
+            const uint32_t slices = sliced && plan->host_copy ? 4 : 1;
+            static_assert(DJ_SEGS % 4 == 0, "slices of whole segments");
+            if (slices > 1 && !c->copy_stream)
+                JN_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
+            for (uint32_t k = 0; k < slices; k++) {
+                ps.w = segs / slices;
+                ps.lo = k * ps.w;
+                JN_TRY(join_once(MODE_EMIT, plan->dev, ps));
+                if (slices == 1) break;
+                const uint64_t from = ps.at[ps.lo], to = k + 1 < slices ? ps.at[ps.lo + ps.w] : normal;
+                cudaEvent_t e;  // the slice's copy begins when it is written, on the copy stream
+                JN_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+                cudaEventRecord(e, c->stream);
+                cudaStreamWaitEvent(c->copy_stream, e, 0);
+                if (to > from)
+                    JN_CUDA(c, cudaMemcpyAsync(*plan->user_out + from, plan->dev + from, (to - from) * sizeof(jn_pair),
+                                               cudaMemcpyDefault, c->copy_stream));
+                if (k + 1 == slices) {  // the run ends when its last copy has landed
+                    cudaEventRecord(e, c->copy_stream);
+                    cudaStreamWaitEvent(c->stream, e, 0);
+                    copied = normal;
+                }
+                cudaEventDestroy(e);
+            }
         }
     }
     if (heavy_pairs > 0) {
@@ -1090,6 +1144,12 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
                       (const uint64_t*)PR.hoff, (const RW*)PS.hrows, (const uint64_t*)PS.hoff,
                       (const uint64_t*)hpoff, (const uint64_t*)hchp, HV_MAX, (uint64_t)CE_PAIRS, normal,
                       plan->dev));
+    }
+    if (copied) {
+        if (heavy_pairs > 0)
+            JN_CUDA(c, cudaMemcpyAsync(*plan->user_out + copied, plan->dev + copied, heavy_pairs * sizeof(jn_pair),
+                                       cudaMemcpyDefault, c->stream));
+        plan->copied = true;
     }
     JN_TRY(out_finish(c, total, *plan));
     return JN_OK;

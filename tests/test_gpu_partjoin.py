@@ -54,3 +54,32 @@ def test_partition_join(ctx, nr, ns, domain, bits, dt, path, rows):
     finally:
         ctx.set_memory_limit(0)
         ctx.set_tuning(hash_path=0, radix_bits=0, table_rows=0)
+
+
+# Eight segments of pairs in both passes: results past the scratch kept for
+# them and under a memory limit (counted, then written at the segments'
+# places), and, from 2^23 rows on, written in slices that are copied to a host
+# buffer as they are finished, frequent keys' pairs behind them.
+@pytest.mark.parametrize("algo", [jn.jn_hash, jn.jn_sort_merge])
+@pytest.mark.parametrize("n,domain,host", [(300000, 60000, False), (300000, 60000, True), ((1 << 23) + 5, 1 << 24, True)])
+def test_segments(ctx, algo, n, domain, host):
+    r = datagen.uniform_keys(n, 0, domain, 97, 0)
+    s = datagen.uniform_keys(n, 0, domain, 97, 1)
+    if n > 1 << 20:
+        r[100:30100], s[7:207] = 12345, 12345
+    exp = O.hash_join(r.numpy(), s.numpy(), np.arange(n, dtype=np.int32), np.arange(n, dtype=np.int32))
+    R, S = jn.table(r.to(DEV)), jn.table(s.to(DEV))
+    out = torch.empty((exp.shape[0] + 3, 2), dtype=torch.int32, pin_memory=True) if host else None
+    ctx.set_tuning(radix_bits=10 if n < 1 << 20 else 13)
+    try:
+        for limit in (0, 8 << 30):
+            ctx.set_memory_limit(limit)
+            got = algo(ctx, R, S, out=out)
+            got = got[: exp.shape[0]].cpu().numpy()
+            word = lambda p: np.sort(np.ascontiguousarray(p).view(np.int64).ravel())
+            assert np.array_equal(word(got), word(exp))
+            if out is not None:
+                out.zero_()
+    finally:
+        ctx.set_memory_limit(0)
+        ctx.set_tuning(radix_bits=0)
