@@ -2,9 +2,9 @@
 
 Default workload: the large equi-join, R = S = 2^28 rows of (int32 key,
 int32 payload = row id), keys Zipf(theta) over 2^28 values (theta = 0 by
-default), run as the pre-filtered, radix-partitioned hash join with the exact
-count pass and one exact output allocation.  A step is one full jn_hash call
-(partition with the pre-filter, count pass, scan, allocation, emit); the
+default), run as the pre-filtered, radix-partitioned hash join with one
+exact output allocation.  A step is one full jn_hash call (partition with the
+pre-filter, the pairs found and counted, allocation, their copy); the
 partition path is the one the library takes (regions by default: one radix
 pass, then one block per region splits it and keeps the pre-filter's bitmap
 slice of the region in shared memory).
@@ -1078,11 +1078,11 @@ def main():
                 "traffic": None,
                 "algorithmic_bytes_per_launch": abytes[dom] / max(kern[dom]["launches_per_step"], 1)}
     if w["kind"] == "nlj":
-        # compare-bound: every launch evaluates all n_R x n_S pairs.  The peak is
-        # the SMs' issue rate (4 schedulers x 32 lanes per SM per clock) over the
+        # compare-bound: a pass evaluates all n_R x n_S pairs.  The peak is the
+        # SMs' issue rate (4 schedulers x 32 lanes per SM per clock) over the
         # thread instructions the kernel issues per pair, as ncu counted them
         # (smsp__thread_inst_executed.sum / pairs, 4K x 64K two-column band
-        # predicate, profiles/nested_loop_64Kx1M.md)
+        # predicate of this workload, too wide to screen)
         sm_mhz = pk.get("sm_max_mhz", 2070.0)
         nsm = torch.cuda.get_device_properties(local).multi_processor_count
         cand = [k for k in ("nlj_count", "nlj_emit") if k in kern]
@@ -1091,7 +1091,7 @@ def main():
             dk = max(cand, key=lambda k: kern[k]["ms_per_step"])
             ipp = NLJ_THREAD_INSTR_PER_PAIR[dk]
             peak = nsm * 4 * 32 * sm_mhz * 1e6 / ipp
-            a = nr * ns / (kern[dk]["avg_launch_ms"] * 1e-3)
+            a = nr * ns / (kern[dk]["ms_per_step"] * 1e-3)
             roof = {"bound": "alu", "kernel": dk, "achieved": a, "peak": peak, "unit": "pair evaluations/s",
                     "frac": a / peak, "traffic": None, "thread_instructions_per_pair": ipp,
                     "peak_kind": "issue rate: %d SMs x 128 lanes x %.0f MHz / %.2f thread instructions per pair "

@@ -10,8 +10,8 @@
  *   - the GPU entry points take the two tables and their sizes, as
  *     Join_GPU(T', S', NB_T, NB_S) of Algorithm 1 and GPU_theta_join(S, T) of
  *     Algorithm 3 do;
- *   - the output is sized exactly by a count pass before it is written, in
- *     place of the Cartesian-product bound of Eq. (rsize) (Sec. 3.3.3).
+ *   - the output is sized exactly before it is allocated (the pairs are
+ *     counted, or found once and kept in scratch), in place of the Cartesian-product bound of Eq. (rsize) (Sec. 3.3.3).
  * R is the build side (the paper's T, "the smaller table", Sec. 2.3) and S the
  * probe side.
  *
@@ -196,8 +196,8 @@ const char* jn_version(void);
 
 /* ------------------------------------------------------------ joins --- */
 
-/* Exact result size of a join without writing pairs (the count pass that
- * replaces Eq. (rsize)'s estimate, Sec. 3.3.3).
+/* Exact result size of a join without writing pairs (the exact count
+ * that replaces Eq. (rsize)'s estimate, Sec. 3.3.3).
  *   algo JN_ALGO_HASH : equality on key (pred must be NULL or op_a = JN_EQ
  *                       with no second conjunct);
  *   algo JN_ALGO_NLJ  : any jn_pred;
@@ -218,7 +218,7 @@ jn_status jn_aggregate(jn_ctx* ctx, int32_t algo, const jn_table* R, const jn_ta
 
 /* Output convention of the three joins:
  *   *out == NULL : the library allocates exactly *n_out pairs of device memory
- *                  (one allocation, after the count pass) and stores the
+ *                  (one allocation, once they are counted) and stores the
  *                  pointer in *out; release it with jn_free.  capacity is ignored.
  *   *out != NULL : a caller buffer of `capacity` pairs, device or host memory.
  *                  The kernels write 8-byte aligned device buffers (and, with
@@ -263,10 +263,11 @@ jn_status jn_hash(jn_ctx* ctx, const jn_table* R, const jn_table* S,
 
 /* Equi sort-merge join: the third category of join algorithms in Sec. 2.3
  * (sort, then walk the tables in order), beside the nested-loop and hash
- * joins the paper builds.  The pre-filter, partitioning, frequent-key path,
- * count pass and exact allocation are those of jn_hash; within a partition
- * each chunk of R rows is sorted by key in shared memory and every S row
- * finds its run of equal keys by binary search.  Same arguments, result and
+ * joins the paper builds.  The pre-filter, partitioning, frequent-key path
+ * and exact allocation are those of the partitioned jn_hash; within a
+ * partition each chunk of R rows is sorted in shared memory (int32 keys in
+ * the order of their hashes) and every S row finds its run of equal keys by
+ * binary search.  Same arguments, result and
  * errors as jn_hash. */
 jn_status jn_sort_merge(jn_ctx* ctx, const jn_table* R, const jn_table* S,
                         jn_pair** out, uint64_t capacity, uint64_t* n_out);
@@ -298,11 +299,12 @@ typedef struct {
  * memory, and *n_out receives the total).  first[i] and pairs[i] (host,
  * count words each) receive where join i's pairs start and how many there
  * are: they are out[first[i] .. first[i] + pairs[i]).  The equi-joins of a
- * batch share every phase (one radix pass over all their tables, one count
- * pass and one emit pass over a single work queue of (join, partition)
- * items), and so do its band joins (one range pass, one count pass and one
- * emit pass over (join, group) items).  Every join is counted before the
- * single exact output allocation; with tuning.graphs on, each phase is
+ * batch share every phase, and so do its band joins: those with a smaller
+ * side of at most 2^22 rows (and, bands, few candidates a row) one build and
+ * one probe of all their tables or indexes; the others one radix or range
+ * pass, one count pass and one emit pass over a single work queue of (join,
+ * partition or group) items.  Every join is counted before the single exact
+ * output allocation; with tuning.graphs on, each phase of the latter is
  * replayed as a CUDA graph.  This is the batched form of the
  * Reducer = grid hierarchy of Sec. 3.3.4: many small joins fill the GPU
  * together instead of one launch sequence each. */
@@ -374,7 +376,7 @@ jn_status jn_autotune_batch(jn_ctx* ctx, int32_t count, const jn_join* joins, jn
  * CUDA stream, so the work of several requests overlaps on the device.
  * Small requests (|R| + |S| < coalesce_rows) waiting at the same time are
  * run together as one jn_batch (at most max_batch of them); larger requests
- * run alone after an exact count pass and wait until their scratch estimate
+ * run alone after an exact count and wait until their scratch estimate
  * plus exact output fits memory_budget next to the outputs still held, as
  * long as another request is running (see jn_server_wait_any).
  * Tables registered with the server stay resident on the device.  The paper
@@ -447,16 +449,16 @@ jn_status jn_server_stats_get(jn_server* s, jn_server_stats* out);
 
 /* ------------------------------------------------------- introspection --- */
 
-/* Admission.  Every join finds its exact result size (the count pass) before
- * it allocates its output.  At that point a context
+/* Admission.  Every join finds its exact result size before it
+ * allocates its output.  At that point a context
  *   - with a memory limit (bytes, 0 = none) refuses a run whose output plus
  *     the scratch it holds exceeds the limit: JN_ERR_OOM, nothing written,
  *     *n_out = the exact pair count;
  *   - with an admission hook calls it with the output bytes it is about to
  *     allocate (0 when the caller supplied device memory) and the scratch
  *     bytes it holds; any status but JN_OK stops the run with that status the
- *     same way.  The hook runs on the calling thread, between the count and
- *     the emit pass, and must not call into the same context.
+ *     same way.  The hook runs on the calling thread, before the
+ *     output is allocated, and must not call into the same context.
  * This is how a caller admits work by exact bytes without a separate count
  * pass (jn_server uses it). */
 typedef jn_status (*jn_admit_fn)(void* user, uint64_t out_bytes, uint64_t scratch_bytes);

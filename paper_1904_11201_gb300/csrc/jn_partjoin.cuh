@@ -21,8 +21,8 @@
 // for three (emit) or four (count, aggregate) on an SM: they cover each
 // other's staging and barriers.  One S row at a time per thread beats two to
 // four with fewer blocks.  Measured on GB300, 2^28 x 2^28 uniform int32 rows:
-// count 1.42 ms (1.65 with k_hash_join), checksum 2.49 (4.22), pairs 4.82
-// with the copy (1.65 + 3.24); 2^26 x 2^26, unique R keys, half matching:
+// count 1.42 ms (1.65 with the kernel it replaced), checksum 2.49 (4.22), pairs
+// 4.82 with the copy (1.65 + 3.24); 2^26 x 2^26, unique R keys, half matching:
 // count 0.29 (0.44), checksum 0.42 (1.08), pairs 0.52 (0.44 + 0.77); int64:
 // 0.74 (0.95), 0.90 (2.07), 1.19 (0.95 + 2.86).
 #pragma once

@@ -1,5 +1,5 @@
 // Partitioned equi hash join (Sec. 3.3.2) with Algorithm 1's pre-filter
-// (Sec. 3.1) and an exact count pass in place of Eq. (rsize) (Sec. 3.3.3).
+// (Sec. 3.1) and an exact count in place of Eq. (rsize) (Sec. 3.3.3).
 //
 // Pipeline on one stream (R = build side, S = probe side):
 //   1. presence: one read of each key column sets a bit per key in the
@@ -12,11 +12,11 @@
 //      the pass-1 output.  Partition p = top (b1 + b2) hash bits; the pair of
 //      passes plays the role of the shuffle on join_key / alpha.
 //   4. work items (partition, R chunk); the join kernel builds a shared-memory
-//      hash table on the R chunk, probes it with the partition's S rows and
-//      keeps the pairs it finds in scratch (jn_partjoin.cuh).
-//   5. one exact allocation (the total is one 8-byte read-back) and one copy.
-//      The sort-merge join counts per item in step 4, scans the counts to
-//      output offsets, and joins a second time to write the pairs there.
+//      hash table on the R chunk (jn_partjoin.cuh) or sorts it
+//      (jn_sortjoin.cuh), looks up the partition's S rows and keeps the pairs
+//      it finds in scratch.
+//   5. one exact allocation (the counts are one read-back) and one copy.  Pairs
+//      that were only counted are found again and written in place.
 #include <vector>
 
 #include "jn_algos.h"
@@ -919,7 +919,7 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
         HashDigit d1{32 - b1, (uint32_t)(F1 - 1)};
         JN_TRY(region ? region_all(d1) : pass_all(d1));
     }
-    // ---- 4. work items and the count pass ----
+    // ---- 4. work items and the join ----
     const int table_rows = cap;
     if (!sort_merge && !heavy && tu.table_rows == 0) {
         // no larger a table than the partitions need (an eighth more than their
@@ -1024,7 +1024,7 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
                       PS.view(), (const uint64_t*)iprefix, P, cap, idesc));
         const int cm = mode == MODE_AGG ? MODE_AGG : MODE_COUNT;
         if (sort_merge) {
-            // every R chunk sorted by key once, into a copy the count and emit passes read
+            // every R chunk sorted once, into a copy that the join reads
             JN_TRY(s.get(&rsorted, (size_t)R.n + HJ_PAD));
             auto sort = [&](auto kso, bool narrow) -> jn_status {
                 const size_t sms = SortJoinSmem<K>::sort_bytes(cap, narrow);
@@ -1092,7 +1092,7 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     info.heavy_pairs = heavy_pairs;
     info.cartesian_bound = h[15] + heavy_pairs;  // the frequent keys' cross products are exact
     if (mode != MODE_EMIT) return JN_OK;
-    // ---- 5. exact allocation and the emit pass ----
+    // ---- 5. exact allocation; the pairs to their places ----
     // kept pairs that did not fit, or that a limit wants for the output
     if (!found.fits || (c->mem_limit && c->scratch_bytes + total * sizeof(jn_pair) > c->mem_limit)) {
         ss.release();

@@ -569,7 +569,7 @@ def jn_nested_loop_noalloc(R: TableRef, S: TableRef, pr: Pred = None, out=None, 
 
 
 def jn_autotune(ctx: Context, algo: int, R: TableRef, S: TableRef, pr: Pred = None) -> dict:
-    """Times candidate tunings through the count pass; applies and returns the fastest."""
+    """Times candidate tunings on the caller's inputs; applies and returns the fastest."""
     t = Tuning()
     st = load().jn_autotune(ctx.handle, algo, ctypes.byref(R.t), ctypes.byref(S.t),
                             ctypes.byref(pr) if pr is not None else None, ctypes.byref(t))
