@@ -973,19 +973,6 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     // 2^24 1.61 (1.73), 2^26 5.15 (5.71), 2^28 19.6 (22.0)
     const bool sliced = mode == MODE_EMIT && segs > 1 && rows >= (1u << 23) && plan->user_out && *plan->user_out &&
                         !is_device_pointer(*plan->user_out);
-    if (mode == MODE_EMIT && nitems && !sliced && !c->admit) {
-        // random keys on both sides match a surviving row 1.6 times; under a
-        // limit that counts scratch only with place for as many bytes of output
-        // (2^28 x 2^28 random int32 rows: 10.7 ms, 11.3 counted first and then
-        // written)
-        room = (rows + rows / 4 * 3) / segs + 4096;
-        if (c->mem_limit && c->scratch_bytes + 2 * segs * room * sizeof(jn_pair) > c->mem_limit) {
-            room = 0;
-        } else if (ss.get(&staged, segs * room) != JN_OK) {
-            c->err.clear();
-            room = 0;
-        }
-    }
     auto join_once = [&](int m, jn_pair* to, const PairSegs& ps) -> jn_status {
         // as many blocks as are resident, a multiple of the launch's segments
         auto grid = [&](uint64_t resident) {
@@ -1014,11 +1001,6 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
                       c->d_err);
     };
     PairSegs ps{};
-    ps.segs = ps.w = segs;
-    for (uint32_t i = 0; i < segs; i++) {
-        ps.at[i] = i * room;
-        ps.cap[i] = room;
-    }
     if (nitems) {
         JN_TRY(launch(c, K_ITEMS, k_item_desc, dim3((unsigned)ceil_div(nitems, 256)), dim3(256), 0, PR.view(),
                       PS.view(), (const uint64_t*)iprefix, P, cap, idesc));
@@ -1035,6 +1017,38 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             if constexpr (sizeof(K) == 8) JN_TRY(sort(k_sort_chunks<K>, false));
             else if (b >= SJ_IDX) JN_TRY(sort(k_sort_chunks32<uint32_t>, true));
             else JN_TRY(sort(k_sort_chunks32<uint64_t>, false));
+        }
+        if (mode == MODE_EMIT && !sliced && !c->admit) {
+            // random keys on both sides match a surviving row 1.6 times; under a
+            // limit that counts scratch only with place for as many bytes of output
+            // (2^28 x 2^28 random int32 rows: 10.7 ms, 11.3 counted first and then
+            // written)
+            room = (rows + rows / 4 * 3) / segs + 4096;
+            if (nitems >= 4096 && rows >= (1u << 23)) {
+                // many pairs a row: one work item in 64 is counted first, so that a
+                // large join does not keep pairs only to find them again (2^28 x
+                // 2^28 rows, Zipf 0.5, 1.3e9 pairs: 16.7 ms, 28.8 without; the
+                // sample takes 0.03 ms)
+                PairSegs one{};
+                one.segs = 64;
+                one.w = 1;
+                JN_TRY(join_once(MODE_COUNT, nullptr, one));
+                uint64_t seen;
+                JN_TRY(read_back(c, reinterpret_cast<const uint64_t*>(&small->lines[0].total), &seen, 1));
+                JN_TRY(zero(c, &small->lines[0].total, 8));
+                if (64 * seen > segs * room) room = 0;
+            }
+            if (room && c->mem_limit && c->scratch_bytes + 2 * segs * room * sizeof(jn_pair) > c->mem_limit) {
+                room = 0;
+            } else if (room && ss.get(&staged, segs * room) != JN_OK) {
+                c->err.clear();
+                room = 0;
+            }
+        }
+        ps.segs = ps.w = segs;
+        for (uint32_t i = 0; i < segs; i++) {
+            ps.at[i] = i * room;
+            ps.cap[i] = room;
         }
         JN_TRY(join_once(room ? MODE_EMIT : cm, staged, ps));
     }

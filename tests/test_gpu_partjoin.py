@@ -61,7 +61,8 @@ def test_partition_join(ctx, nr, ns, domain, bits, dt, path, rows):
 # places), and, from 2^23 rows on, written in slices that are copied to a host
 # buffer as they are finished, frequent keys' pairs behind them.
 @pytest.mark.parametrize("algo", [jn.jn_hash, jn.jn_sort_merge])
-@pytest.mark.parametrize("n,domain,host", [(300000, 60000, False), (300000, 60000, True), ((1 << 23) + 5, 1 << 24, True)])
+@pytest.mark.parametrize("n,domain,host", [(300000, 60000, False), (300000, 60000, True), ((1 << 23) + 5, 1 << 24, True),
+                                           ((1 << 23) + 5, 1 << 22, False)])
 def test_segments(ctx, algo, n, domain, host):
     r = datagen.uniform_keys(n, 0, domain, 97, 0)
     s = datagen.uniform_keys(n, 0, domain, 97, 1)
