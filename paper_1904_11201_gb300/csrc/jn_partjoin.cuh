@@ -126,7 +126,8 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     Item d{};
     if (first_item < nitems) d = items[first_item];
     for (uint64_t it = first_item; it < nitems; it += step) {
-        const int rn = d.rn, sn = d.sn;
+        const int rn = d.rn;
+        const uint32_t sn = (uint32_t)d.sn;  // below 2^31: a row number and a round past it fit 32 bits
         const uint64_t lo = (d.rbeg * sizeof(R)) & ~15ull;
         // bytes of rows [beg, beg + n), widened to 16-byte boundaries
         auto span = [](uint64_t beg, int n) {
@@ -151,10 +152,10 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         // the thread's first S rows come in while the table is built
         const R* sp = srows + d.sbeg;
         R x[PU];
-        auto load = [&](int j0) {
+        auto load = [&](uint32_t j0) {
 #pragma unroll
             for (int u = 0; u < PU; u++) {
-                const int j = j0 + u * PJ_T + tid;
+                const uint32_t j = j0 + u * PJ_T + tid;
                 if (j < sn) x[u] = sp[j];
             }
         };
@@ -244,7 +245,7 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
             __syncthreads();
         }
         // ---- probe ----
-        for (int j0 = 0; j0 < sn; j0 += PU * PJ_T) {
+        for (uint32_t j0 = 0; j0 < sn; j0 += PU * PJ_T) {
             R y[PU];
 #pragma unroll
             for (int u = 0; u < PU; u++) y[u] = x[u];

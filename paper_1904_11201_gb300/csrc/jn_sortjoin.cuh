@@ -308,6 +308,7 @@ k_sort_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     for (uint64_t it = ps.first(); it < nitems; it += next) {
         const Item d = items[it];
         const uint32_t rn = (uint32_t)d.rn;
+        const uint32_t sn = (uint32_t)d.sn;  // below 2^31: a row number and a round past it fit 32 bits
         for (uint32_t i = tid; i < rn; i += SJ_T) {  // the chunk, sorted by key
             const Row<K, false> x = rrows[d.rbeg + i];
             s_k[sj_swz(i)] = (U)x.key;
@@ -337,18 +338,18 @@ k_sort_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         while (2 * top <= rn) top <<= 1;
         // a warp takes groups of 256 consecutive S rows
         const Row<K, false>* sp = srows + d.sbeg;
-        for (int g = (tid >> 5) * 32 * PER; g < d.sn; g += SJ_T * PER) {
+        for (uint32_t g = (tid >> 5) * 32 * PER; g < sn; g += SJ_T * PER) {
             U q[PER];
             int32_t spay[PER];
             uint32_t lo[PER], m[PER];
 #pragma unroll
             for (int e = 0; e < PER; e++) {
-                const int j = g + e * 32 + lane;
+                const uint32_t j = g + e * 32 + lane;
                 lo[e] = 0;
                 m[e] = 0;
                 q[e] = 0;
                 spay[e] = 0;
-                if (j < d.sn) {
+                if (j < sn) {
                     const Row<K, false> x = sp[j];
                     q[e] = sj_ord(x.key, bits);
                     spay[e] = x.pay;
@@ -365,7 +366,7 @@ k_sort_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
             uint32_t sum = 0;
 #pragma unroll
             for (int e = 0; e < PER; e++) {
-                if (g + e * 32 + lane < d.sn && lo[e] < rn && s_k[sj_swz(lo[e])] == q[e]) {
+                if (g + e * 32 + lane < sn && lo[e] < rn && s_k[sj_swz(lo[e])] == q[e]) {
                     // the run's length: by doubling, then by halving
                     uint32_t a = 1, step = 1;
                     while (lo[e] + a < rn && s_k[sj_swz(lo[e] + a)] == q[e]) {

@@ -107,6 +107,9 @@ __global__ void k_item_desc(PartView rv, PartView sv, const uint64_t* __restrict
     items[it] = d;
 }
 
+// Staged chunks of sn S rows (up to 2^31 - 1 of them, so the sum is unsigned).
+__device__ __forceinline__ int s_chunks(int sn) { return (int)(((uint32_t)sn + HJ_SCH - 1) / HJ_SCH); }
+
 // Starts the copy of rows [beg, beg + n) into `g` (widened to 16 bytes);
 // returns the byte offset of row `beg` inside the staged span.
 template <typename R>
@@ -213,7 +216,7 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     // S-chunk stream: chunk q of this block sits in buffer q & 1; thread 0
     // stages chunks ahead (producer), every thread consumes them in order.
     uint64_t p_it = it;  // producer: item and chunk of the next chunk to stage
-    int p_sc = 0, p_nsc = (d.sn + HJ_SCH - 1) / HJ_SCH;
+    int p_sc = 0, p_nsc = s_chunks(d.sn);
     uint64_t p_sbeg = d.sbeg;
     int p_sn = d.sn;
     bool p_valid = true;
@@ -230,7 +233,7 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
                 const Item x = items[p_it];
                 p_sbeg = x.sbeg;
                 p_sn = x.sn;
-                p_nsc = (x.sn + HJ_SCH - 1) / HJ_SCH;
+                p_nsc = s_chunks(x.sn);
                 p_sc = 0;
             }
         }
@@ -361,7 +364,7 @@ k_hash_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
         // ---- probe with every S chunk of the partition ----
         unsigned long long acc = 0;
         const uint64_t ibase = MODE == MODE_EMIT ? item_off[it] : 0;
-        const int nsc = (d.sn + HJ_SCH - 1) / HJ_SCH;
+        const int nsc = s_chunks(d.sn);
         for (int sc = 0; sc < nsc; sc++) {
             const uint32_t b = qc & 1, ph = (qc >> 1) & 1;
             if (__syncthreads_or(!mbar_wait(&bar_s[b], ph, err))) {
