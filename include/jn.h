@@ -487,6 +487,14 @@ int32_t jn_pointer_is_device(const void* p);            /* 1 if p is device (or 
  * range or no context), JN_ERR_CUDA. */
 jn_status jn_selftest_wait(jn_ctx* ctx, uint32_t polls, int32_t arrive, uint64_t* elapsed_ns);
 
+/* Diagnostic of what a call does on a device with little memory left (not
+ * part of the join method).  From now on a device allocation of this context
+ * that would take the scratch it holds past `bytes` fails on the host, as the
+ * allocator does when the device is full; 0 ends this.  Unlike a memory
+ * limit, which refuses a run, this lets a call fall back to ways that need
+ * less. */
+jn_status jn_selftest_memory(jn_ctx* ctx, uint64_t bytes);
+
 #ifdef __cplusplus
 }
 #endif

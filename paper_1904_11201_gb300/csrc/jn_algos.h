@@ -30,10 +30,23 @@ struct OutPlan {
     bool lib_alloc = false;      // library allocated the result
     bool mapped = false;         // caller buffer is page-locked host memory written in place
     bool copied = false;         // the run already copied the pairs to the caller's host buffer
+    bool admitted = false;       // the limit and the hook have let the run pass: they are asked once
+    bool no_memory = false;      // the output's allocation failed
 };
 
 // Sizes the output for `m` pairs (allocating or checking the caller buffer).
 jn_status out_prepare(jn_ctx* c, Scratch& s, uint64_t m, OutPlan& plan);
+// The same for a run that keeps its pairs in scratch: where the output finds no
+// memory beside them, give_up() releases them (true: it had some) and the
+// allocation is tried once more; the run then writes its pairs in a second pass.
+template <typename F>
+jn_status out_prepare_or(jn_ctx* c, Scratch& s, uint64_t m, OutPlan& plan, F give_up) {
+    const jn_status st = out_prepare(c, s, m, plan);
+    if (st != JN_ERR_OOM || !plan.no_memory || !give_up()) return st;
+    c->err.clear();
+    JN_CUDA(c, cudaStreamSynchronize(c->stream));  // the released memory can take another shape
+    return out_prepare(c, s, m, plan);
+}
 // Copies to a host buffer when needed and publishes the result.
 jn_status out_finish(jn_ctx* c, uint64_t m, OutPlan& plan);
 

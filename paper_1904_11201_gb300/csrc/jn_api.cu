@@ -30,17 +30,21 @@ jn_status out_prepare(jn_ctx* c, Scratch& s, uint64_t m, OutPlan& plan) {
     plan.lib_alloc = false;
     const jn_pair* mapped =
         user && (c->tune.host_io & 2) ? static_cast<const jn_pair*>(host_mapped(user)) : nullptr;
-    {
+    plan.no_memory = false;
+    if (!plan.admitted) {
         const bool dev_out =
             user != nullptr && (m == 0 || m > plan.capacity || mapped || is_device_pointer(user));
         JN_TRY(admit(c, m, dev_out ? 0 : m * sizeof(jn_pair), plan));
+        plan.admitted = true;
     }
     if (user == nullptr) {
         plan.lib_alloc = true;
         plan.dev = nullptr;
         if (m > 0) {
             void* p = nullptr;
-            JN_TRY(dalloc(c, &p, m * sizeof(jn_pair)));
+            const jn_status st = dalloc(c, &p, m * sizeof(jn_pair));
+            plan.no_memory = st == JN_ERR_OOM;
+            if (st != JN_OK) return st;
             plan.dev = static_cast<jn_pair*>(p);
         }
         return JN_OK;
@@ -62,7 +66,9 @@ jn_status out_prepare(jn_ctx* c, Scratch& s, uint64_t m, OutPlan& plan) {
         return JN_OK;
     }
     plan.host_copy = true;
-    return s.get(&plan.dev, m);
+    const jn_status st = s.get(&plan.dev, m);
+    plan.no_memory = st == JN_ERR_OOM;
+    return st;
 }
 
 jn_status out_finish(jn_ctx* c, uint64_t m, OutPlan& plan) {
@@ -240,9 +246,10 @@ static jn_status run(jn_ctx* c, int algo, const jn_table* R, const jn_table* S, 
     return JN_OK;
 }
 
+// direct: joins may run without partitioning; *direct then tells whether one did.
 template <typename K>
-static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair** out, uint64_t capacity,
-                             uint64_t* n_out, uint64_t* first, uint64_t* pairs, bool count_only) {
+static jn_status batch_parts(jn_ctx* c, int count, const jn_join* joins, jn_pair** out, uint64_t capacity,
+                             uint64_t* n_out, uint64_t* first, uint64_t* pairs, bool count_only, bool* direct) {
     Scratch s(c);
     // the batch's parts: equi-joins with a table small enough to stay in L2
     // and the others, band joins likewise; each part runs as one
@@ -250,9 +257,11 @@ static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair
     std::vector<int> part[PARTS];
     for (int i = 0; i < count; i++) {
         const int64_t nr = joins[i].R.n, ns = joins[i].S.n;
-        part[joins[i].band >= 0 ? (band_direct_takes(c, nr, ns) ? 2 : 3) : batch_direct_takes(c, nr, ns) ? 0 : 1]
+        part[joins[i].band >= 0 ? (*direct && band_direct_takes(c, nr, ns) ? 2 : 3)
+                                : *direct && batch_direct_takes(c, nr, ns) ? 0 : 1]
             .push_back(i);
     }
+    *direct = !part[0].empty() || !part[2].empty();
     std::vector<Cols<K>> cr[PARTS], cs[PARTS];
     std::vector<int> bops[PARTS];
     std::vector<int64_t> bbands[PARTS];
@@ -344,7 +353,11 @@ static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair
     uint64_t at = 0;
     for (int k = 0; k < PARTS; k++) {
         if (!run[k]) continue;
-        JN_TRY(run[k]->emit(c, plan.dev + at));
+        const jn_status st = run[k]->emit(c, plan.dev + at);
+        if (st != JN_OK) {
+            if (plan.lib_alloc) dfree(c, plan.dev);
+            return st;
+        }
         at += run[k]->total;
     }
     publish();
@@ -355,6 +368,23 @@ static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair
     JN_TRY(read_back(c, d_small, &dummy, 0));  // reports a device wait that ran out
     c->info.result = total;
     return JN_OK;
+}
+
+template <typename K>
+static jn_status batch_typed(jn_ctx* c, int count, const jn_join* joins, jn_pair** out, uint64_t capacity,
+                             uint64_t* n_out, uint64_t* first, uint64_t* pairs, bool count_only) {
+    bool direct = true;
+    const jn_status st =
+        batch_parts<K>(c, count, joins, out, capacity, n_out, first, pairs, count_only, &direct);
+    if (st != JN_ERR_OOM || !direct) return st;
+    // tables, indexes and kept pairs left too little of the device for the
+    // other joins or the output: every join partitioned, which keeps nothing
+    // (direct joins are not taken under a limit or a hook, so neither refused)
+    c->err.clear();
+    c->info = jn_run_info();
+    JN_CUDA(c, cudaStreamSynchronize(c->stream));  // the released memory can take another shape
+    direct = false;
+    return batch_parts<K>(c, count, joins, out, capacity, n_out, first, pairs, count_only, &direct);
 }
 
 }  // namespace jnx

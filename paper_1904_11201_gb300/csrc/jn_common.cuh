@@ -89,6 +89,7 @@ struct jn_ctx {
     cudaEvent_t copied_r = nullptr;      // ... and every column of its first table (or NULL)
     cudaEvent_t copied_all = nullptr;    // every host column of this run has landed (or NULL)
     uint64_t scratch_bytes = 0;  // bytes held by live Scratch sets
+    uint64_t test_memory = 0;    // self-test: allocations past this many scratch bytes fail (0 = none)
     uint64_t mem_limit = 0;      // admission: output + scratch bound (0 = none)
     jn_admit_fn admit = nullptr;
     void* admit_user = nullptr;

@@ -41,6 +41,10 @@ jn_status cuda_fail(jn_ctx* c, cudaError_t e, const char* what) {
 }
 
 jn_status dalloc(jn_ctx* c, void** p, size_t bytes) {
+    if (c->test_memory && c->scratch_bytes + bytes > c->test_memory) {
+        *p = nullptr;
+        return fail(c, JN_ERR_OOM, "device allocation: past the self-test's memory");
+    }
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
     if (e != cudaSuccess) {
         *p = nullptr;
@@ -503,6 +507,12 @@ jn_status jn_last_run_info(const jn_ctx* c, jn_run_info* info) {
 uint64_t jn_launch_count(const jn_ctx* c) { return c ? c->launches_total : 0; }
 
 int32_t jn_pointer_is_device(const void* p) { return p && is_device_pointer(p) ? 1 : 0; }
+
+jn_status jn_selftest_memory(jn_ctx* c, uint64_t bytes) {
+    if (!c) return JN_ERR_INVALID;
+    c->test_memory = bytes;
+    return JN_OK;
+}
 
 jn_status jn_selftest_wait(jn_ctx* c, uint32_t polls, int32_t arrive, uint64_t* elapsed_ns) {
     if (!c || polls < 1 || polls > (1u << 20) || (arrive != 0 && arrive != 1)) return JN_ERR_INVALID;

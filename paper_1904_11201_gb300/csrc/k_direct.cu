@@ -76,7 +76,18 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
     if (MODE != MODE_EMIT) return JN_OK;
     // a table no longer needed, or the scratch the pairs did not fit
     (done ? s : ss).release();
-    JN_TRY(out_prepare(c, ss, total, *plan));
+    const jn_status st = out_prepare(c, ss, total, *plan);
+    if (st == JN_ERR_OOM && plan->no_memory) {
+        // no memory for the output beside the table or the kept pairs: the
+        // partitioned join, which can do with less
+        c->err.clear();
+        *taken = false;
+        ss.release();
+        s.release();
+        JN_CUDA(c, cudaStreamSynchronize(c->stream));  // the released memory can take another shape
+        return JN_OK;
+    }
+    if (st != JN_OK) return st;
     if (total && done && plan->host_copy && segs == 1) {
         // straight to the caller's buffer
         JN_CUDA(c, cudaMemcpyAsync(*plan->user_out, staged, total * sizeof(jn_pair), cudaMemcpyDefault, c->stream));

@@ -1115,7 +1115,12 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
         ss.release();
         room = 0;
     }
-    JN_TRY(out_prepare(c, s, total, *plan));
+    JN_TRY(out_prepare_or(c, s, total, *plan, [&] {
+        const bool kept = room != 0;
+        ss.release();
+        room = 0;
+        return kept;
+    }));
     uint64_t copied = 0;  // pairs that are on their way to the caller's buffer
     if (normal > 0) {
         if (room && found.fits) {

@@ -572,9 +572,14 @@ jn_status run_nlj(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, const jn_pred& 
     info.prefilter = 0;
     info.cartesian_bound = pairs;  // every pair is compared
     if (mode != MODE_EMIT) return JN_OK;
-    const bool done = h[0] <= cap;
+    bool done = h[0] <= cap;
     if (!done) ss.release();
-    JN_TRY(out_prepare(c, ss, h[0], *plan));
+    JN_TRY(out_prepare_or(c, s, h[0], *plan, [&] {
+        const bool kept = done && cap;
+        ss.release();
+        done = done && !cap;
+        return kept;
+    }));
     if (h[0] && done) {
         // straight to the caller's buffer, host memory included
         JN_CUDA(c, cudaMemcpyAsync(plan->host_copy ? *plan->user_out : plan->dev, staged, h[0] * sizeof(jn_pair),

@@ -280,7 +280,16 @@ jn_status star_direct(jn_ctx* c, const jn_table* R, const jn_table* S1, const jn
     (done ? s : ss).release();  // the tables, or the scratch the triples did not fit
     jn_triple *user = *out, *dev = nullptr;
     bool copy_back = false;
-    JN_TRY(star_output(c, ss, m, user, capacity, n_out, &dev, &copy_back));
+    const jn_status st = star_output(c, ss, m, user, capacity, n_out, &dev, &copy_back);
+    if (st == JN_ERR_OOM) {  // no memory for the output beside the tables or the kept triples: the two joins
+        c->err.clear();
+        *taken = false;
+        ss.release();
+        s.release();
+        JN_CUDA(c, cudaStreamSynchronize(c->stream));  // the released memory can take another shape
+        return JN_OK;
+    }
+    if (st != JN_OK) return st;
     if (m && done) {
         JN_TRY((direct_gather<int32_t, 3>(c, K_STAR, staged, segs, cap, r, dev)));
     } else if (m) {

@@ -849,11 +849,18 @@ jn_status run_theta(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int op, int64
             info.cartesian_bound = run->candidates;
             if (mode != MODE_EMIT) return JN_OK;
             Scratch s(c);
-            JN_TRY(out_prepare(c, s, run->total, *plan));
-            JN_TRY(run->emit(c, plan->dev));
-            return out_finish(c, run->total, *plan);
+            const jn_status so = out_prepare(c, s, run->total, *plan);
+            if (so == JN_OK) {
+                JN_TRY(run->emit(c, plan->dev));
+                return out_finish(c, run->total, *plan);
+            }
+            if (so != JN_ERR_OOM || !plan->no_memory) return so;
+            // no memory for the output beside the index and the kept pairs
+            run.reset();
+            JN_CUDA(c, cudaStreamSynchronize(c->stream));  // the released memory can take another shape
+        } else if (st != JN_OK && st != JN_ERR_OOM) {
+            return st;
         }
-        if (st != JN_OK && st != JN_ERR_OOM) return st;
         c->err.clear();  // too full a device or too many candidates: partitioned
     }
     if (band >= 0) return run_theta_t<K, true>(c, R, S, op, band, mode, plan, res);

@@ -166,6 +166,7 @@ _SIGS = {
     "jn_last_run_info": (ctypes.c_int, [_P, ctypes.POINTER(RunInfo)]),
     "jn_launch_count": (ctypes.c_uint64, [_P]),
     "jn_pointer_is_device": (ctypes.c_int32, [_P]),
+    "jn_selftest_memory": (ctypes.c_int, [_P, ctypes.c_uint64]),
     "jn_selftest_wait": (ctypes.c_int, [_P, ctypes.c_uint32, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint64)]),
 }
 
@@ -596,6 +597,11 @@ def jn_batch_count(ctx: Context, joins) -> list:
     cnt = (ctypes.c_uint64 * max(n, 1))()
     _check(ctx, load().jn_batch_count(ctx.handle, n, arr, cnt, None))
     return [int(cnt[i]) for i in range(n)]
+
+
+def jn_selftest_memory(ctx: Context, nbytes: int):
+    """Device allocations of the context past nbytes of scratch fail (0: none do)."""
+    _check(ctx, load().jn_selftest_memory(ctx.handle, nbytes))
 
 
 def jn_selftest_wait(ctx: Context, polls: int, arrive: bool):
