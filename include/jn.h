@@ -495,6 +495,12 @@ jn_status jn_selftest_wait(jn_ctx* ctx, uint32_t polls, int32_t arrive, uint64_t
  * less. */
 jn_status jn_selftest_memory(jn_ctx* ctx, uint64_t bytes);
 
+/* Diagnostic of a call that fails half way: the n-th kernel launch of this
+ * context from now is not made and its call returns JN_ERR_CUDA, on the host
+ * alone (the device runs what was queued before and the context stays
+ * usable); 0 ends this. */
+jn_status jn_selftest_launches(jn_ctx* ctx, uint64_t n);
+
 #ifdef __cplusplus
 }
 #endif

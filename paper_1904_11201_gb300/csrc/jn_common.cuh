@@ -90,6 +90,7 @@ struct jn_ctx {
     cudaEvent_t copied_all = nullptr;    // every host column of this run has landed (or NULL)
     uint64_t scratch_bytes = 0;  // bytes held by live Scratch sets
     uint64_t test_memory = 0;    // self-test: allocations past this many scratch bytes fail (0 = none)
+    uint64_t test_launches = 0;  // self-test: the launch after this many fails (0 = none)
     uint64_t mem_limit = 0;      // admission: output + scratch bound (0 = none)
     jn_admit_fn admit = nullptr;
     void* admit_user = nullptr;
@@ -157,6 +158,8 @@ template <typename Kern, typename... Args>
 jn_status launch(jn_ctx* c, int kid, Kern kern, dim3 grid, dim3 block, size_t smem,
                  Args... args) {
     if (grid.x == 0 || grid.y == 0 || grid.z == 0) return JN_OK;
+    if (c->test_launches && --c->test_launches == 0)
+        return fail(c, JN_ERR_CUDA, "kernel launch: refused by the self-test");
     if (smem > 0) ensure_smem(reinterpret_cast<const void*>(kern), smem);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c->profiling) {

@@ -514,6 +514,12 @@ jn_status jn_selftest_memory(jn_ctx* c, uint64_t bytes) {
     return JN_OK;
 }
 
+jn_status jn_selftest_launches(jn_ctx* c, uint64_t n) {
+    if (!c) return JN_ERR_INVALID;
+    c->test_launches = n;
+    return JN_OK;
+}
+
 jn_status jn_selftest_wait(jn_ctx* c, uint32_t polls, int32_t arrive, uint64_t* elapsed_ns) {
     if (!c || polls < 1 || polls > (1u << 20) || (arrive != 0 && arrive != 1)) return JN_ERR_INVALID;
     c->err.clear();

@@ -723,6 +723,19 @@ static jn_status region_partition(jn_ctx* c, Scratch& s, const Cols<K>& R, const
     return JN_OK;
 }
 
+// Copies of finished slices on the copy stream.  A run that fails with some of
+// them queued waits for them: they read scratch it is about to release and
+// write the caller's buffer.
+struct SliceCopies {
+    jn_ctx* c;
+    cudaEvent_t e = nullptr;
+    bool queued = false;  // copies that the run's stream does not wait for yet
+    ~SliceCopies() {
+        if (queued) cudaStreamSynchronize(c->copy_stream);
+        if (e) cudaEventDestroy(e);
+    }
+};
+
 template <typename K>
 jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutPlan* plan,
                    RunResult* res, bool sort_merge) {
@@ -1139,25 +1152,28 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             static_assert(DJ_SEGS % 4 == 0, "slices of whole segments");
             if (slices > 1 && !c->copy_stream)
                 JN_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
+            SliceCopies sc{c};
             for (uint32_t k = 0; k < slices; k++) {
                 ps.w = segs / slices;
                 ps.lo = k * ps.w;
                 JN_TRY(join_once(MODE_EMIT, plan->dev, ps));
                 if (slices == 1) break;
                 const uint64_t from = ps.at[ps.lo], to = k + 1 < slices ? ps.at[ps.lo + ps.w] : normal;
-                cudaEvent_t e;  // the slice's copy begins when it is written, on the copy stream
-                JN_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-                cudaEventRecord(e, c->stream);
-                cudaStreamWaitEvent(c->copy_stream, e, 0);
-                if (to > from)
+                // the slice's copy begins when it is written, on the copy stream
+                if (!sc.e) JN_CUDA(c, cudaEventCreateWithFlags(&sc.e, cudaEventDisableTiming));
+                JN_CUDA(c, cudaEventRecord(sc.e, c->stream));
+                JN_CUDA(c, cudaStreamWaitEvent(c->copy_stream, sc.e, 0));
+                if (to > from) {
+                    sc.queued = true;
                     JN_CUDA(c, cudaMemcpyAsync(*plan->user_out + from, plan->dev + from, (to - from) * sizeof(jn_pair),
                                                cudaMemcpyDefault, c->copy_stream));
+                }
                 if (k + 1 == slices) {  // the run ends when its last copy has landed
-                    cudaEventRecord(e, c->copy_stream);
-                    cudaStreamWaitEvent(c->stream, e, 0);
+                    JN_CUDA(c, cudaEventRecord(sc.e, c->copy_stream));
+                    JN_CUDA(c, cudaStreamWaitEvent(c->stream, sc.e, 0));
+                    sc.queued = false;
                     copied = normal;
                 }
-                cudaEventDestroy(e);
             }
         }
     }

@@ -167,6 +167,7 @@ _SIGS = {
     "jn_launch_count": (ctypes.c_uint64, [_P]),
     "jn_pointer_is_device": (ctypes.c_int32, [_P]),
     "jn_selftest_memory": (ctypes.c_int, [_P, ctypes.c_uint64]),
+    "jn_selftest_launches": (ctypes.c_int, [_P, ctypes.c_uint64]),
     "jn_selftest_wait": (ctypes.c_int, [_P, ctypes.c_uint32, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint64)]),
 }
 
@@ -602,6 +603,11 @@ def jn_batch_count(ctx: Context, joins) -> list:
 def jn_selftest_memory(ctx: Context, nbytes: int):
     """Device allocations of the context past nbytes of scratch fail (0: none do)."""
     _check(ctx, load().jn_selftest_memory(ctx.handle, nbytes))
+
+
+def jn_selftest_launches(ctx: Context, n: int):
+    """The context's n-th kernel launch from now fails on the host (0: none does)."""
+    _check(ctx, load().jn_selftest_launches(ctx.handle, n))
 
 
 def jn_selftest_wait(ctx: Context, polls: int, arrive: bool):
