@@ -27,6 +27,7 @@
 // rows, join by join.  Pairs go to rooms of scratch (several per large join,
 // for their cursors' sake) through per-warp buffers, and one copy puts them in
 // the exact allocation.
+#include <math.h>
 #include <string.h>
 
 #include <algorithm>
@@ -47,6 +48,11 @@ constexpr uint64_t BD_MOST = 48;   // candidates a row past which a probe stops
 constexpr int BD_SAMPLE_P = 512;   // rows sampled for the estimate: of the probing table,
 constexpr int BD_SAMPLE_B = 4096;  // and of the built one, in BD_SPARTS parts
 constexpr int BD_SPARTS = 64;      // (the estimate takes 9 us; 13 in 16 parts)
+constexpr int BD_CHECK_B = 1024, BD_CPARTS = 16;  // and, of the built one, by k_band_ranges
+// Rows of the index a row meets past which nothing is built.  What puts that
+// many into a few buckets fills few of the partitioned join's groups too:
+// counts with far values, 28 and 128 rows met, take 1.0 and 1.15 times its time.
+constexpr double BD_MEET = 128;
 constexpr uint64_t BD_ROOM = 1ull << 30;  // pairs of room at most (8 GB)
 constexpr int BD_ROOMS = DJ_SEGS;  // rooms of a large join
 
@@ -59,7 +65,8 @@ struct BandJoin {
     int64_t bn, pn;
     uint64_t row0;      // build rows of the joins before this one
     uint64_t off0;      // first of its offsets: `buckets` and one behind
-    uint64_t most;      // candidates past which it stops
+    uint64_t most;      // candidates past which its probe stops
+    uint64_t most_hits; // hits past which nothing is built
     long long band;
     uint32_t buckets;   // a power of two
     int32_t op;         // built row's a `op` probing row's a
@@ -77,7 +84,9 @@ struct BandRange {
 struct BandMark {
     unsigned long long hi, nlo;  // max of ord(k), max of ~ord(k)
     unsigned long long work;     // candidates met
-    unsigned long long stop;     // too many
+    unsigned long long stop;     // too many, or too many to come
+    unsigned long long hits;     // sampled pairs whose rows meet in the index
+    unsigned long long pad;
 };
 
 struct BandRoom {
@@ -169,22 +178,52 @@ k_band_bounds(BandBatch<K> b) {
     }
 }
 
-template <typename K>
-__global__ void k_band_ranges(BandBatch<K> b) {
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < b.n; j += gridDim.x * blockDim.x) {
-        BandRange r;
-        r.hi = (long long)(b.mark[j].hi ^ (1ull << 63));
-        r.lo = (long long)(~b.mark[j].nlo ^ (1ull << 63));
-        const uint64_t span = (uint64_t)r.hi - (uint64_t)r.lo;
-        r.shift = 0;
-        while (r.shift < 63 && (span >> r.shift) >= (uint64_t)b.joins[j].buckets) r.shift++;
-        r.pad = 0;
-        b.range[j] = r;
-    }
-}
-
 __device__ __forceinline__ uint64_t bd_bucket(const BandRange& r, long long k) {
     return ((uint64_t)k - (uint64_t)r.lo) >> r.shift;
+}
+
+// The joins' ranges (the first of a join's BD_CPARTS blocks), and mark[j].hits +=
+// pairs of sampled rows that meet in the index: the built row lies in a bucket
+// that the other's window touches (a block takes a part of the built sample).  The index pays
+// for these and not for the rows inside the band alone: one value far from the
+// others puts all of them into a few buckets.  A join with more than most_hits
+// is left to the partitioned join before it is built; its rows are what every
+// window's warp scanned before the probe's own limit was seen (2^16 x 2^16 int32
+// rows, one key 300 times further out than the others' range: 0.88 ms, 0.27 now,
+// 0.20 partitioned at once).
+template <typename K>
+__global__ void __launch_bounds__(BD_T)
+k_band_ranges(BandBatch<K> b) {
+    __shared__ uint64_t s_b[BD_CHECK_B / BD_CPARTS];
+    const int j = blockIdx.x / BD_CPARTS, part = blockIdx.x % BD_CPARTS;
+    const uint64_t most_hits = b.joins[j].most_hits;
+    if (part && most_hits == ~0ull) return;
+    BandRange g;
+    g.hi = (long long)(b.mark[j].hi ^ (1ull << 63));
+    g.lo = (long long)(~b.mark[j].nlo ^ (1ull << 63));
+    const uint64_t width = (uint64_t)g.hi - (uint64_t)g.lo;
+    const uint32_t buckets = b.joins[j].buckets;
+    // the smallest shift with width >> shift < buckets, a power of two
+    g.shift = width >= buckets ? (64 - __clzll((long long)width)) - (31 - __clz((int)buckets)) : 0;
+    g.pad = 0;
+    if (part == 0 && threadIdx.x == 0) b.range[j] = g;
+    if (most_hits == ~0ull) return;
+    const BandJoin<K> d = b.joins[j];
+    const int nb = (int)min(d.bn, (int64_t)BD_CHECK_B), np = (int)min(d.pn, (int64_t)BD_SAMPLE_P);
+    const int b0 = part * (BD_CHECK_B / BD_CPARTS), cnt = min(BD_CHECK_B / BD_CPARTS, nb - b0);
+    if (cnt <= 0) return;  // the whole block
+    for (int i = threadIdx.x; i < cnt; i += BD_T) s_b[i] = bd_bucket(g, (long long)d.bk[(int64_t)(b0 + i) * d.bn / nb]);
+    __syncthreads();
+    unsigned int m = 0;
+    for (int p = threadIdx.x; p < np; p += BD_T) {
+        const Interval<K> iv = band_interval<K>(d.pk[(int64_t)p * d.pn / np], d.band);
+        const long long first = (long long)iv.lo, last = (long long)(K)((decltype(iv.span))iv.lo + iv.span);
+        if (last < g.lo || first > g.hi) continue;
+        const uint64_t lo = bd_bucket(g, max(first, g.lo)), span = bd_bucket(g, min(last, g.hi)) - lo;
+        for (int i = 0; i < cnt; i++) m += s_b[i] - lo <= span;
+    }
+    m = warp_sum(m);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(&b.mark[j].hits, (unsigned long long)m);
 }
 
 template <typename K>
@@ -193,6 +232,10 @@ k_band_count(BandBatch<K> b) {
     const uint64_t tiles = b.btiles[b.n];
     for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int j = find_segment(b.btiles, b.n, t);
+        if (b.mark[j].hits > b.joins[j].most_hits) {
+            if (threadIdx.x == 0) b.mark[j].stop = 1;
+            continue;
+        }
         const BandJoin<K> d = b.joins[j];
         const BandRange r = b.range[j];
         const int64_t r0 = (int64_t)(t - b.btiles[j]) * BD_ROWS, end = min(d.bn, r0 + BD_ROWS);
@@ -207,6 +250,7 @@ k_band_place(BandBatch<K> b) {
     const uint64_t tiles = b.btiles[b.n];
     for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int j = find_segment(b.btiles, b.n, t);
+        if (b.mark[j].stop) continue;
         const BandJoin<K> d = b.joins[j];
         const BandRange r = b.range[j];
         const int64_t r0 = (int64_t)(t - b.btiles[j]) * BD_ROWS, end = min(d.bn, r0 + BD_ROWS);
@@ -440,6 +484,13 @@ struct BandDirectRun : BandDirect {
             d.buckets = 64;
             while (d.buckets < (uint64_t)d.bn) d.buckets <<= 1;
             d.most = BD_MOST * (uint64_t)d.pn + 65536;
+            // sampled pairs that meet where a row meets BD_MEET, with room for
+            // chance; small joins meet few rows at worst
+            const double meet = d.bn ? BD_MEET * (double)std::min(d.pn, (int64_t)BD_SAMPLE_P) *
+                                           (double)std::min(d.bn, (int64_t)BD_CHECK_B) / (double)d.bn
+                                     : 0;
+            const bool small = (double)d.bn * (double)d.pn < (double)(1u << 28);
+            d.most_hits = small ? ~0ull : (uint64_t)(meet + 3 * sqrt(meet) + 4);
             d.room0 = (uint32_t)rooms.size();
             d.rooms = d.pn >= (1 << 21) ? BD_ROOMS : 1;
             const uint64_t cap =
@@ -566,7 +617,7 @@ struct BandDirectRun : BandDirect {
         auto kl = k_band_place<K>;
         auto kp = k_band_probe<K, MODE>;
         JN_TRY(launch(c, K_MINMAX, kb, grid((const void*)kb, btiles), dim3(BD_T), 0, b));
-        JN_TRY(launch(c, K_MINMAX, k_band_ranges<K>, dim3((unsigned)ceil_div((uint64_t)n, 128)), dim3(128), 0, b));
+        JN_TRY(launch(c, K_MINMAX, k_band_ranges<K>, dim3(BD_CPARTS * (unsigned)n), dim3(BD_T), 0, b));
         JN_TRY(launch(c, K_BAND_BUILD, kc, grid((const void*)kc, btiles), dim3(BD_T), 0, b));
         JN_TRY(scan_u32_u32(c, b.count, b.off, offs));
         JN_TRY(launch(c, K_BAND_BUILD, kl, grid((const void*)kl, btiles), dim3(BD_T), 0, b));
