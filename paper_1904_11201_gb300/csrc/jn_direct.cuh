@@ -63,7 +63,8 @@ struct DirectLine {
     unsigned long long first;   // [0]: star join: pairs of the first join
     unsigned long long cursor;  // [0]: words placed in `runs`
     unsigned int dup;           // [0]: some key has several build rows (emit)
-    unsigned int pad[23];
+    unsigned int longs;         // [0]: parts of long runs left to k_direct_long
+    unsigned int pad[22];
 };
 struct DirectSmall {
     DirectLine lines[DJ_SEGS];
@@ -352,6 +353,33 @@ __device__ __forceinline__ bool dj_single(bool dup, uint32_t m) {
     return DirectSlot<K, MODE_EMIT>::COUNTS_ASIDE ? !dup : m == 1;
 }
 
+// A part of a long run: the pairs of one probe row with n payloads at src, to
+// dst.  The row's warp reserves their place and k_direct_long writes them, a
+// warp to a part, so frequent keys load the whole device wherever their probe
+// rows lie.  A warp that wrote such runs itself, those of a sorted column one
+// after the other, was all that ran: 2^14 x 2^14 rows, a key 4096 times in one
+// and in 256 neighbouring rows of the other, 0.81 ms (int64).
+struct LongRun {
+    int2* dst;
+    const int32_t* src;
+    uint32_t n_swap;  // n, and in the top bit whether the payloads at src are S's
+    int32_t pay;      // the probe row's
+};
+constexpr uint32_t DJ_LONG = 128;       // rows of a key past which its run is a long one
+constexpr uint32_t DJ_LONG_PART = 1024;
+static_assert(DJ_LONG_PART > DJ_LONG, "a run of m > DJ_LONG rows has at most m / DJ_LONG parts");
+
+static __global__ void __launch_bounds__(256)
+k_direct_long(const LongRun* __restrict__ longs, const unsigned int* __restrict__ count) {
+    const uint32_t n = *count, lane = threadIdx.x & 31;
+    for (uint32_t w = (blockIdx.x * 256 + threadIdx.x) >> 5; w < n; w += gridDim.x * 8) {
+        const LongRun r = longs[w];
+        const uint32_t m = r.n_swap & 0x7fffffffu;
+        const bool swap = r.n_swap >> 31;
+        for (uint32_t e = lane; e < m; e += 32) r.dst[e] = swap ? make_int2(r.pay, r.src[e]) : make_int2(r.src[e], r.pay);
+    }
+}
+
 // A warp's results on their way out: they collect in shared memory and leave
 // DJ_BUF at a time, as one reservation of the output cursor and coalesced
 // stores.  No warp waits for another: with a reservation per block and round
@@ -368,6 +396,10 @@ struct WarpOut {
     T* out;
     unsigned long long cap;
     uint32_t fill;
+    // long runs are listed here (NULL: written by the warp).  Room for one part
+    // per DJ_LONG results that can be reserved always suffices.
+    LongRun* longs = nullptr;
+    unsigned int* nlongs = nullptr;
     // where the warp's next n results start; false: they do not fit
     __device__ __forceinline__ bool reserve(unsigned long long n, unsigned long long* at) const {
         unsigned long long a = 0;
@@ -463,8 +495,22 @@ __device__ __forceinline__ void dj_probe_rows(const K* __restrict__ key, const i
                         st_pair(o + e, swap ? pp[u] : bp, swap ? bp : pp[u]);
                     }
                 }
-                // a longer run is written by the whole warp, 32 pairs at a time
-                for (unsigned lanes = __ballot_sync(0xffffffffu, m[u] > 4); lanes; lanes &= lanes - 1) {
+                // long runs are listed, in parts
+                const uint32_t parts =
+                    wo.longs && m[u] > DJ_LONG ? (m[u] + DJ_LONG_PART - 1) / DJ_LONG_PART : 0u;
+                if (__any_sync(0xffffffffu, parts)) {
+                    const uint32_t before = warp_incl_scan(parts) - parts;
+                    uint32_t q = 0;
+                    if (lane == 31) q = atomicAdd(wo.nlongs, before + parts);
+                    q = __shfl_sync(0xffffffffu, q, 31) + before;
+                    for (uint32_t e = 0; e < parts; e++) {
+                        const uint32_t at0 = e * DJ_LONG_PART;
+                        wo.longs[q + e] = LongRun{reinterpret_cast<int2*>(o) + at0, t.runs + v[u] + at0,
+                                                  min(DJ_LONG_PART, m[u] - at0) | (uint32_t)swap << 31, pp[u]};
+                    }
+                }
+                // a shorter one is written by the whole warp, 32 pairs at a time
+                for (unsigned lanes = __ballot_sync(0xffffffffu, m[u] > 4 && !parts); lanes; lanes &= lanes - 1) {
                     const int src = __ffs(lanes) - 1;
                     const uint32_t lm = __shfl_sync(0xffffffffu, m[u], src);
                     const uint32_t lv = __shfl_sync(0xffffffffu, v[u], src);
@@ -493,14 +539,15 @@ __device__ __forceinline__ void dj_probe_rows(const K* __restrict__ key, const i
 template <typename K, int MODE>
 __global__ void __launch_bounds__(DJ_T, JN_DJ_MINB)
 k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int swap,
-               DirectSmall* __restrict__ small, jn_pair* __restrict__ out, uint32_t segs, unsigned long long cap) {
+               DirectSmall* __restrict__ small, jn_pair* __restrict__ out, uint32_t segs, unsigned long long cap,
+               LongRun* __restrict__ longs) {
     constexpr int TILE = DJ_T * DJ_U;
     using Out = WarpOut<2>;
     __shared__ int2 s_buf[MODE == MODE_EMIT ? DJ_T / 32 : 1][MODE == MODE_EMIT ? Out::ROOM : 1];
     const uint32_t seg = blockIdx.x % segs;
     out += seg * cap;
     Out wo{MODE == MODE_EMIT ? s_buf[threadIdx.x >> 5] : nullptr, &small->lines[seg].total,
-           reinterpret_cast<int2*>(out), cap, 0};
+           reinterpret_cast<int2*>(out), cap, 0, longs, &small->lines[0].longs};
     unsigned long long acc = 0, csum = 0;
     dj_probe_rows<K, MODE>(key, pay, (int64_t)blockIdx.x * TILE, n, (int64_t)gridDim.x * TILE, t, swap, wo, acc, csum);
     if (MODE == MODE_EMIT) {
@@ -639,12 +686,15 @@ struct DirectResult {
     DirectCounts counts;
     uint64_t total = 0, chk = 0, first = 0;
     bool fits = true;  // every segment's results fit its room
+    bool dup = false;  // some build key has several rows
+    uint32_t longs = 0;
 };
 // Queues the counters' copy to the host; after the stream is synchronised,
 // direct_parse reads them.
 constexpr int DJ_HWORD = 16;  // where they land in the context's pinned words
+constexpr int DJ_LINE_WORDS = 5;  // words of a line that matter here
 inline jn_status direct_fetch(jn_ctx* c, const DirectSmall* small, uint32_t segs) {
-    constexpr int W = 4;  // words of a line that matter here
+    constexpr int W = DJ_LINE_WORDS;
     static_assert(DJ_HWORD + W * DJ_SEGS < 63, "the last pinned word is read_back's error word");
     JN_CUDA(c, cudaMemcpy2DAsync(c->h_small + DJ_HWORD, W * 8, small, sizeof(DirectLine), W * 8, segs,
                                  cudaMemcpyDeviceToHost, c->stream));
@@ -653,18 +703,25 @@ inline jn_status direct_fetch(jn_ctx* c, const DirectSmall* small, uint32_t segs
 inline void direct_parse(const jn_ctx* c, uint32_t segs, uint64_t cap, DirectResult* r) {
     const uint64_t* h = c->h_small + DJ_HWORD;
     for (uint32_t i = 0; i < segs; i++) {
-        r->counts.n[i] = h[4 * i];
+        r->counts.n[i] = h[DJ_LINE_WORDS * i];
         r->total += r->counts.n[i];
         r->fits &= r->counts.n[i] <= cap;
     }
     r->chk = h[1];
     r->first = h[2];
+    r->dup = (h[4] & 0xffffffffu) != 0;
+    r->longs = (uint32_t)(h[4] >> 32);
 }
 inline jn_status direct_result(jn_ctx* c, const DirectSmall* small, uint32_t segs, uint64_t cap, DirectResult* r) {
     JN_TRY(direct_fetch(c, small, segs));
     JN_CUDA(c, cudaStreamSynchronize(c->stream));
     direct_parse(c, segs, cap, r);
     return JN_OK;
+}
+
+// Writes the long runs that a probe listed.
+inline jn_status direct_long(jn_ctx* c, const LongRun* longs, const unsigned int* count) {
+    return launch(c, K_DIRECT_PROBE, k_direct_long, dim3(8 * (unsigned)c->num_sms), dim3(256), 0, longs, count);
 }
 
 template <typename T, int PER>

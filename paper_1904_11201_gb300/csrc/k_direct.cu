@@ -9,11 +9,6 @@
 
 namespace jnx {
 
-// Pairs past which an emitting run is left to the partitioned join: many
-// times the rows, so frequent keys carry it, whose cross products that join
-// writes as dense tiles spread over the whole device.
-static uint64_t direct_most_pairs(uint64_t rows) { return 8 * rows + (1u << 20); }
-
 template <typename K, int MODE>
 static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutPlan* plan, RunResult* res,
                              bool* taken) {
@@ -26,11 +21,13 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
     const DirectStage sg(np);
     uint32_t segs = MODE == MODE_EMIT ? sg.segs : 1;
     uint64_t cap = MODE == MODE_EMIT ? sg.cap : 0;
+    // kept pairs, and the long runs among them
+    auto keep_bytes = [&](uint64_t pairs) { return pairs * sizeof(jn_pair) + (pairs / DJ_LONG + 1) * sizeof(LongRun); };
     if (c->mem_limit || c->admit) {
         // a run admitted by its bytes holds no more scratch here than the
         // partitioned join would (two copies of the rows of both tables)
         const uint64_t most = 2 * (sizeof(K) == 4 ? 8 : 16) * (nb + np);
-        if (head + lay.bytes() + segs * cap * sizeof(jn_pair) > most) cap = 0;
+        if (head + lay.bytes() + keep_bytes(segs * cap) > most) cap = 0;
         if (head + lay.bytes() > most) return JN_OK;
     }
     Scratch s(c);
@@ -41,9 +38,15 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
         return JN_OK;
     }
     Scratch ss(c);
-    if (cap && ss.get(&staged, segs * cap) != JN_OK) {
+    LongRun* longs = nullptr;
+    unsigned char* kept = nullptr;
+    if (cap && ss.get(&kept, keep_bytes(segs * cap)) != JN_OK) {
         c->err.clear();
         cap = 0;
+    }
+    if (cap) {
+        staged = reinterpret_cast<jn_pair*>(kept);
+        longs = reinterpret_cast<LongRun*>(kept + segs * cap * sizeof(jn_pair));
     }
     DirectSmall* small = reinterpret_cast<DirectSmall*>(mem);
     JN_TRY(zero(c, mem, head + lay.zeroed()));
@@ -56,12 +59,11 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
     const uint64_t tiles = ceil_div(np, DJ_T * DJ_U);
     const dim3 g((unsigned)std::min<uint64_t>(tiles, (uint64_t)std::max(per, 1) * c->num_sms));
     JN_TRY(launch(c, K_DIRECT_PROBE, kp, g, dim3(DJ_T), 0, P.key, P.pay, P.n, t, swap ? 1 : 0, small, staged, segs,
-                  (unsigned long long)cap));
+                  (unsigned long long)cap, longs));
     DirectResult r;
     JN_TRY(direct_result(c, small, segs, cap, &r));
     const uint64_t total = r.total;
     const bool done = r.fits;
-    if (MODE == MODE_EMIT && !done && total > direct_most_pairs(nb + np)) return JN_OK;
     *taken = true;
     jn_run_info& info = c->info;
     res->count = total;
@@ -74,6 +76,7 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
     info.hash_path = 3;
     info.cartesian_bound = nb * np;
     if (MODE != MODE_EMIT) return JN_OK;
+    if (done && r.longs) JN_TRY(direct_long(c, longs, &small->lines[0].longs));
     // a table no longer needed, or the scratch the pairs did not fit
     (done ? s : ss).release();
     const jn_status st = out_prepare(c, ss, total, *plan);
@@ -95,9 +98,13 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
     } else if (total && done) {
         JN_TRY((direct_gather<uint64_t, 1>(c, K_DIRECT_PROBE, staged, segs, cap, r, plan->dev)));
     } else if (total) {
+        longs = nullptr;  // a run admitted by its bytes takes no more scratch
+        if (r.dup && !c->mem_limit && !c->admit && ss.get(&longs, total / DJ_LONG + 1) != JN_OK) c->err.clear();
         JN_TRY(zero(c, &small->lines[0].total, 8));
+        JN_TRY(zero(c, &small->lines[0].longs, 4));
         JN_TRY(launch(c, K_DIRECT_PROBE, kp, g, dim3(DJ_T), 0, P.key, P.pay, P.n, t, swap ? 1 : 0, small, plan->dev,
-                      1u, (unsigned long long)total));
+                      1u, (unsigned long long)total, longs));
+        if (longs) JN_TRY(direct_long(c, longs, &small->lines[0].longs));
         JN_CUDA(c, cudaStreamSynchronize(c->stream));  // this pass reads the caller's columns
     }
     return out_finish(c, total, *plan);
@@ -160,6 +167,7 @@ struct DirectBatch {
     uint2* where;
     int32_t* runs;
     DirectLine* lines;
+    LongRun* longs;  // long runs of all joins, counted in lines[0]
     __device__ __forceinline__ DirectTab<K, MODE> table(const DirectJoin<K>& d, int j) const {
         using DS = DirectSlot<K, MODE>;
         DirectTab<K, MODE> t;
@@ -224,7 +232,8 @@ k_batch_probe(DirectBatch<K, MODE> b, jn_pair* __restrict__ out, const uint64_t*
             if (cap <= d.cap) continue;  // already written
             cursor = &b.lines[j].chk;    // the first pass's total stays
         }
-        Out wo{MODE == MODE_EMIT ? s_buf[threadIdx.x >> 5] : nullptr, cursor, reinterpret_cast<int2*>(out + at), cap, 0};
+        Out wo{MODE == MODE_EMIT ? s_buf[threadIdx.x >> 5] : nullptr, cursor, reinterpret_cast<int2*>(out + at), cap, 0,
+               b.longs, &b.lines[0].longs};
         unsigned long long acc = 0, csum = 0;
         dj_probe_rows<K, MODE>(d.pkey, d.ppay, row, min(d.pn, row + DB_ROWS), DJ_T * DJ_U, b.table(d, j), d.swap, wo,
                                acc, csum);
@@ -310,6 +319,7 @@ struct DirectBatchRun : BatchRun {
             JN_TRY(s->get(&b.where, rows));
             JN_TRY(s->get(&b.runs, rows * (DS::COUNTS_ASIDE ? 2 : 1)));
             JN_TRY(s->get(&staged, stage));
+            if (stage) JN_TRY(s->get(&b.longs, stage / DJ_LONG + 1));
         }
         b.joins = d_joins;
         b.btiles = d_bt;
@@ -336,8 +346,10 @@ struct DirectBatchRun : BatchRun {
                 if ((st = launch(c, K_DIRECT_BUILD, kr, g, dim3(DJ_T), 0, b, 1)) != JN_OK) break;
             }
             auto kp = k_batch_probe<K, MODE>;
-            st = launch(c, K_DIRECT_PROBE, kp, grid(c, (const void*)kp, ptiles), dim3(DJ_T), 0, b, staged,
-                        (const uint64_t*)nullptr);
+            if ((st = launch(c, K_DIRECT_PROBE, kp, grid(c, (const void*)kp, ptiles), dim3(DJ_T), 0, b, staged,
+                             (const uint64_t*)nullptr)) != JN_OK)
+                break;
+            if (b.longs) st = direct_long(c, b.longs, &b.lines[0].longs);
         } while (0);
         if (st != JN_OK) {
             gp.abort();
@@ -378,8 +390,12 @@ struct DirectBatchRun : BatchRun {
                           (const uint64_t*)d_off, (const uint64_t*)(d_words + n), n, reinterpret_cast<uint64_t*>(out)));
             if (!fits) {
                 auto kp = k_batch_probe<K, MODE>;
+                b.longs = nullptr;
+                if (s->get(&b.longs, total / DJ_LONG + 1) != JN_OK) c->err.clear();
+                JN_TRY(zero(c, &b.lines[0].longs, 4));
                 JN_TRY(launch(c, K_DIRECT_PROBE, kp, grid(c, (const void*)kp, ptiles), dim3(DJ_T), 0, b, out,
                               (const uint64_t*)d_off));
+                if (b.longs) JN_TRY(direct_long(c, b.longs, &b.lines[0].longs));
             }
         }
         return JN_OK;
