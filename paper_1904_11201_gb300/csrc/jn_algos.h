@@ -63,10 +63,11 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
                    RunResult* res, bool sort_merge = false);
 
 // The direct join (jn_direct.cuh), when it suits the tables and the tuning:
-// *taken false = nothing was done, the partitioned join is to run.
+// *taken false = nothing was done, the partitioned join is to run (*repeats:
+// because the build keys have several rows).
 template <typename K>
 jn_status run_direct(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutPlan* plan, RunResult* res,
-                     bool* taken);
+                     bool* taken, bool* repeats);
 
 // A batch of joins run as one: prepare() (all passes up to the exact
 // counts) fills total and the per-join offsets; emit() writes the pairs to

@@ -31,6 +31,8 @@
 
 #include <algorithm>
 
+#include <algorithm>
+
 #include "jn_algos.h"
 #include "jn_common.cuh"
 
@@ -64,7 +66,8 @@ struct DirectLine {
     unsigned long long cursor;  // [0]: words placed in `runs`
     unsigned int dup;           // [0]: some key has several build rows (emit)
     unsigned int longs;         // [0]: parts of long runs left to k_direct_long
-    unsigned int pad[22];
+    unsigned int left;          // [0]: nothing was done (dj_left)
+    unsigned int pad[21];
 };
 struct DirectSmall {
     DirectLine lines[DJ_SEGS];
@@ -172,6 +175,124 @@ __device__ __forceinline__ uint32_t dj_claim(const DirectTab<K, MODE>& t, K k) {
     return t.zero_slot();  // not reached: the table has twice the slots of its rows
 }
 
+// ------------------------------------------------------- repeated keys --
+// Repeated build keys cost the direct join a run per key: counts, starts and
+// payloads, each a random access to a table or an array (int32 rows, ms for a
+// build of 2^22: 0.11 without repeats, 0.31 with).  Where that decides between
+// the direct and the partitioned join, the rows of one hash in 2^shift are
+// counted first, 1024 to 2048 of them, and their keys.  The build's kernels
+// read the counts themselves: no host round trip (25 us here) in between.
+constexpr int DUP_SLOTS = 4096;   // per table
+constexpr int DUP_ROWS = 2048;    // rows per tile
+struct DupCount {
+    unsigned long long rows, keys;
+};
+template <typename K>
+struct DupTable {
+    const K* key;
+    int64_t n;
+    int shift, pad;
+};
+// Tables by value, with their tiles' prefix.
+constexpr int DUP_MANY = 32;
+template <typename K>
+struct DupTables {
+    DupTable<K> t[DUP_MANY];
+    uint32_t tiles[DUP_MANY + 1];
+    int n;
+    void add(const K* key, int64_t rows) {  // n < DUP_MANY
+        int shift = 0;
+        while ((rows >> shift) >= 2048) shift++;
+        t[n] = DupTable<K>{key, rows, shift, 0};
+        tiles[n + 1] = tiles[n] + (uint32_t)ceil_div((uint64_t)rows, DUP_ROWS);
+        n++;
+    }
+};
+template <typename K>
+inline size_t dup_bytes(int n) {  // counts, then slots: start as zeros
+    return ((size_t)n * (sizeof(DupCount) + DUP_SLOTS * sizeof(K)) + 255) & ~(size_t)255;
+}
+
+// Not the tables' and partitions' hash: the keys looked at lie all over them.
+__device__ __forceinline__ uint32_t dup_hash(int32_t k) {
+    uint32_t h = (uint32_t)k * 0x2C1B3C6Du;
+    h = (h ^ (h >> 15)) * 0x297A2D39u;
+    return h ^ (h >> 16);
+}
+__device__ __forceinline__ uint32_t dup_hash(int64_t k) {
+    return dup_hash((int32_t)((uint32_t)k ^ (uint32_t)((uint64_t)k >> 32) * 0x9E3779B1u));
+}
+
+// counts[j] of table j; key 0 is left out.
+template <typename K>
+__global__ void __launch_bounds__(256)
+k_dup_sample(const __grid_constant__ DupTables<K> tabs, DupCount* __restrict__ counts) {
+    K* const slots = reinterpret_cast<K*>(counts + tabs.n);
+    const uint32_t ntiles = tabs.tiles[tabs.n];
+    int j = 0;
+    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        while (tabs.tiles[j + 1] <= t) j++;
+        const DupTable<K> d = tabs.t[j];
+        const int64_t r0 = (int64_t)(t - tabs.tiles[j]) * DUP_ROWS, end = min(d.n, r0 + DUP_ROWS);
+        K* tab = slots + (size_t)j * DUP_SLOTS;
+        unsigned int rows = 0, keys = 0;
+        constexpr int U = DUP_ROWS / 256;
+        K k[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int64_t i = r0 + u * 256 + threadIdx.x;
+            k[u] = i < end ? d.key[i] : K(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const uint32_t h = dup_hash(k[u]);
+            if (k[u] == K(0) || (d.shift && h >> (32 - d.shift))) continue;
+            rows++;
+            uint32_t s = h & (DUP_SLOTS - 1);
+            bool known = false;
+            for (int probe = 0; probe < 64 && !known; probe++) {
+                K old = *(volatile K*)(tab + s);
+                if (old == K(0)) {
+                    if (sizeof(K) == 4)
+                        old = (K)atomicCAS(reinterpret_cast<unsigned int*>(tab + s), 0u, (unsigned int)k[u]);
+                    else
+                        old = (K)atomicCAS(reinterpret_cast<unsigned long long*>(tab + s), 0ull,
+                                           (unsigned long long)k[u]);
+                    if (old == K(0)) break;  // a new key
+                }
+                known = old == k[u];
+                s = (s + 1) & (DUP_SLOTS - 1);
+            }
+            keys += !known;
+        }
+        rows = warp_sum(rows);
+        keys = warp_sum(keys);
+        if ((threadIdx.x & 31) == 0 && rows) {
+            atomicAdd(&counts[j].rows, (unsigned long long)rows);
+            atomicAdd(&counts[j].keys, (unsigned long long)keys);
+        }
+    }
+}
+
+template <typename K>
+jn_status dup_sample(jn_ctx* c, const DupTables<K>& tabs, DupCount* counts) {
+    const uint32_t tiles = std::max(tabs.tiles[tabs.n], 1u);
+    return launch(c, K_DIRECT_BUILD, k_dup_sample<K>, dim3(std::min<uint32_t>(tiles, 8 * (uint32_t)c->num_sms)),
+                  dim3(256), 0, tabs, counts);
+}
+
+// A single join is left to the partitioned one: 1.8 rows a key and more.
+__device__ __forceinline__ bool dj_left(const DupCount* dup) { return dup && 5 * dup->rows > 9 * dup->keys; }
+
+// n 16-byte words set to zero by the block's share of a grid.
+__device__ __forceinline__ void dj_zero(uint4* p, uint64_t n) {
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+        p[i] = make_uint4(0, 0, 0, 0);
+}
+static __global__ void __launch_bounds__(256) k_direct_zero(uint4* p, uint64_t n, const DupCount* __restrict__ dup) {
+    if (!dj_left(dup)) dj_zero(p, n);
+}
+
 // Inserts the build rows.  Emit: where[i] = (slot, rank among the key's
 // rows), and the rank-0 row leaves its payload in the slot, which is final
 // when no key has several rows.  use_g: the build side is S.
@@ -220,7 +341,8 @@ __device__ __forceinline__ void dj_insert_rows(const K* __restrict__ key, const 
 template <typename K, int MODE>
 __global__ void __launch_bounds__(DJ_T)
 k_direct_insert(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int use_g,
-                uint2* __restrict__ where, DirectSmall* __restrict__ small) {
+                uint2* __restrict__ where, DirectSmall* __restrict__ small, const DupCount* __restrict__ dup) {
+    if (dj_left(dup)) return;
     dj_insert_rows<K, MODE>(key, pay, (int64_t)blockIdx.x * DJ_T, n, (int64_t)gridDim.x * DJ_T, t, use_g, where,
                             small->lines);
 }
@@ -540,10 +662,14 @@ template <typename K, int MODE>
 __global__ void __launch_bounds__(DJ_T, JN_DJ_MINB)
 k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int swap,
                DirectSmall* __restrict__ small, jn_pair* __restrict__ out, uint32_t segs, unsigned long long cap,
-               LongRun* __restrict__ longs) {
+               LongRun* __restrict__ longs, const DupCount* __restrict__ dup) {
     constexpr int TILE = DJ_T * DJ_U;
     using Out = WarpOut<2>;
     __shared__ int2 s_buf[MODE == MODE_EMIT ? DJ_T / 32 : 1][MODE == MODE_EMIT ? Out::ROOM : 1];
+    if (MODE == MODE_EMIT && dj_left(dup)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) small->lines[0].left = 1;
+        return;
+    }
     const uint32_t seg = blockIdx.x % segs;
     out += seg * cap;
     Out wo{MODE == MODE_EMIT ? s_buf[threadIdx.x >> 5] : nullptr, &small->lines[seg].total,
@@ -649,7 +775,7 @@ struct DirectLayout {
 // Launches of one table's build in `mem` (already zeroed up to lay.zeroed()).
 template <typename K, int MODE>
 jn_status direct_build(jn_ctx* c, const Cols<K>& B, int use_g, const DirectLayout<K, MODE>& lay, unsigned char* mem,
-                       DirectSmall* small, DirectTab<K, MODE>* t) {
+                       DirectSmall* small, DirectTab<K, MODE>* t, const DupCount* dup = nullptr) {
     t->slots = reinterpret_cast<typename DirectTab<K, MODE>::Slot*>(mem);
     t->nb = dj_buckets<K, MODE>((uint64_t)B.n);
     t->counts = reinterpret_cast<uint32_t*>(mem + lay.slots);
@@ -659,7 +785,7 @@ jn_status direct_build(jn_ctx* c, const Cols<K>& B, int use_g, const DirectLayou
     t->dup = &small->lines[0].dup;
     const dim3 g((unsigned)std::min<uint64_t>(ceil_div((uint64_t)B.n, DJ_T), (uint64_t)c->num_sms * 8));
     JN_TRY(launch(c, K_DIRECT_BUILD, k_direct_insert<K, MODE>, g, dim3(DJ_T), 0, B.key, B.pay, B.n, *t, use_g, where,
-                  small));
+                  small, dup));
     if constexpr (MODE == MODE_EMIT) {
         JN_TRY(launch(c, K_DIRECT_BUILD, k_direct_runs<K>, g, dim3(DJ_T), 0, B.n, *t, (const uint2*)where, small));
         JN_TRY(launch(c, K_DIRECT_BUILD, k_direct_place<K>, g, dim3(DJ_T), 0, B.pay, B.n, *t, (const uint2*)where,
@@ -668,17 +794,19 @@ jn_status direct_build(jn_ctx* c, const Cols<K>& B, int use_g, const DirectLayou
     return JN_OK;
 }
 
-// Staged results of a probe of np rows: segments and results per segment.  A
-// join that matches a probe row about once fits (a little more than once, as
-// random keys do); blocks take rows in turn, so segments fill evenly.
+// Staged results of a probe of np rows: segments and results per segment, with
+// room for `quarters` quarters of a result a row.  Blocks take rows in turn, so
+// segments fill evenly.  Pairs past their room are found a second time, so the
+// room is for two rows a key and a little more, as random keys have it (int32,
+// 2^20 x 2^24, two a key: 0.63 ms, 1.02 with five quarters; 0.77 partitioned).
+constexpr uint32_t DJ_ROOM = 9, DJ_ROOM_LEAST = 5;  // quarters
 struct DirectStage {
     uint32_t segs;
     uint64_t cap;
-    explicit DirectStage(uint64_t np) {
+    DirectStage(uint64_t np, uint32_t quarters) {
         segs = np >= (1u << 23) ? DJ_SEGS : 1;
-        cap = (np + np / 4) / segs + 1024;
+        cap = np * quarters / 4 / segs + 1024;
     }
-    uint64_t results() const { return segs * cap; }
 };
 
 // What a probe left in the counters.
@@ -687,12 +815,13 @@ struct DirectResult {
     uint64_t total = 0, chk = 0, first = 0;
     bool fits = true;  // every segment's results fit its room
     bool dup = false;  // some build key has several rows
+    bool left = false;
     uint32_t longs = 0;
 };
 // Queues the counters' copy to the host; after the stream is synchronised,
 // direct_parse reads them.
-constexpr int DJ_HWORD = 16;  // where they land in the context's pinned words
-constexpr int DJ_LINE_WORDS = 5;  // words of a line that matter here
+constexpr int DJ_HWORD = 8;   // where they land in the context's pinned words
+constexpr int DJ_LINE_WORDS = 6;  // words of a line that matter here
 inline jn_status direct_fetch(jn_ctx* c, const DirectSmall* small, uint32_t segs) {
     constexpr int W = DJ_LINE_WORDS;
     static_assert(DJ_HWORD + W * DJ_SEGS < 63, "the last pinned word is read_back's error word");
@@ -711,6 +840,7 @@ inline void direct_parse(const jn_ctx* c, uint32_t segs, uint64_t cap, DirectRes
     r->first = h[2];
     r->dup = (h[4] & 0xffffffffu) != 0;
     r->longs = (uint32_t)(h[4] >> 32);
+    r->left = (h[5] & 0xffffffffu) != 0;
 }
 inline jn_status direct_result(jn_ctx* c, const DirectSmall* small, uint32_t segs, uint64_t cap, DirectResult* r) {
     JN_TRY(direct_fetch(c, small, segs));

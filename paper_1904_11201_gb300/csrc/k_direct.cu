@@ -11,14 +11,14 @@ namespace jnx {
 
 template <typename K, int MODE>
 static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutPlan* plan, RunResult* res,
-                             bool* taken) {
+                             bool* taken, bool* repeats) {
     const bool swap = S.n < R.n;
     const Cols<K>&B = swap ? S : R, &P = swap ? R : S;
     const uint64_t nb = (uint64_t)B.n, np = (uint64_t)P.n;
     const DirectLayout<K, MODE> lay(nb);
     const size_t head = sizeof(DirectSmall);
     static_assert(sizeof(DirectSmall) % 32 == 0, "buckets follow the counters, 32-byte aligned");
-    const DirectStage sg(np);
+    const DirectStage sg(np, DJ_ROOM), less(np, DJ_ROOM_LEAST);
     uint32_t segs = MODE == MODE_EMIT ? sg.segs : 1;
     uint64_t cap = MODE == MODE_EMIT ? sg.cap : 0;
     // kept pairs, and the long runs among them
@@ -27,13 +27,20 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
         // a run admitted by its bytes holds no more scratch here than the
         // partitioned join would (two copies of the rows of both tables)
         const uint64_t most = 2 * (sizeof(K) == 4 ? 8 : 16) * (nb + np);
+        if (head + lay.bytes() + keep_bytes(segs * cap) > most) cap = std::min(cap, less.cap);
         if (head + lay.bytes() + keep_bytes(segs * cap) > most) cap = 0;
         if (head + lay.bytes() > most) return JN_OK;
     }
     Scratch s(c);
     unsigned char* mem = nullptr;
     jn_pair* staged = nullptr;
-    if (s.get(&mem, head + lay.bytes()) != JN_OK) {
+    // Pairs written, 8-byte slots: past 2^21 build rows the table and the runs of
+    // repeated keys leave L2, and with two rows a key the partitioned join is the
+    // faster one (2^22 x 2^24 rows, two a key: 0.81 ms there, 0.91 here; four 1.0
+    // and 1.46; 1.6 rows a key are equal).
+    const bool look = sizeof(K) == 4 && MODE == MODE_EMIT && nb > (1u << 21);
+    const size_t db = look ? dup_bytes<K>(1) : 0;
+    if (s.get(&mem, head + db + lay.bytes()) != JN_OK) {
         c->err.clear();  // a device too full for the table takes the partitioned path
         return JN_OK;
     }
@@ -49,19 +56,32 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
         longs = reinterpret_cast<LongRun*>(kept + segs * cap * sizeof(jn_pair));
     }
     DirectSmall* small = reinterpret_cast<DirectSmall*>(mem);
-    JN_TRY(zero(c, mem, head + lay.zeroed()));
+    JN_TRY(zero(c, mem, head + db + (look ? 0 : lay.zeroed())));
     DirectTab<K, MODE> t;
     JN_TRY(wait_copies(c, true));
-    JN_TRY((direct_build<K, MODE>(c, B, swap ? 1 : 0, lay, mem + head, small, &t)));
+    DupCount* dup = nullptr;
+    if (look) {
+        dup = reinterpret_cast<DupCount*>(mem + head);
+        DupTables<K> tabs{};
+        tabs.add(B.key, B.n);
+        JN_TRY(dup_sample<K>(c, tabs, dup));
+        JN_TRY(launch(c, K_MEMSET, k_direct_zero, dim3(8 * (unsigned)c->num_sms), dim3(256), 0,
+                      reinterpret_cast<uint4*>(mem + head + db), (uint64_t)(lay.zeroed() / 16), (const DupCount*)dup));
+    }
+    JN_TRY((direct_build<K, MODE>(c, B, swap ? 1 : 0, lay, mem + head + db, small, &t, dup)));
     auto kp = k_direct_probe<K, MODE>;
     int per = 0;
     JN_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kp, DJ_T, 0));
     const uint64_t tiles = ceil_div(np, DJ_T * DJ_U);
     const dim3 g((unsigned)std::min<uint64_t>(tiles, (uint64_t)std::max(per, 1) * c->num_sms));
     JN_TRY(launch(c, K_DIRECT_PROBE, kp, g, dim3(DJ_T), 0, P.key, P.pay, P.n, t, swap ? 1 : 0, small, staged, segs,
-                  (unsigned long long)cap, longs));
+                  (unsigned long long)cap, longs, (const DupCount*)dup));
     DirectResult r;
     JN_TRY(direct_result(c, small, segs, cap, &r));
+    if (r.left) {
+        *repeats = true;
+        return JN_OK;
+    }
     const uint64_t total = r.total;
     const bool done = r.fits;
     *taken = true;
@@ -103,7 +123,7 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
         JN_TRY(zero(c, &small->lines[0].total, 8));
         JN_TRY(zero(c, &small->lines[0].longs, 4));
         JN_TRY(launch(c, K_DIRECT_PROBE, kp, g, dim3(DJ_T), 0, P.key, P.pay, P.n, t, swap ? 1 : 0, small, plan->dev,
-                      1u, (unsigned long long)total, longs));
+                      1u, (unsigned long long)total, longs, (const DupCount*)nullptr));
         if (longs) JN_TRY(direct_long(c, longs, &small->lines[0].longs));
         JN_CUDA(c, cudaStreamSynchronize(c->stream));  // this pass reads the caller's columns
     }
@@ -112,19 +132,19 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
 
 template <typename K>
 jn_status run_direct(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutPlan* plan, RunResult* res,
-                     bool* taken) {
-    *taken = false;
+                     bool* taken, bool* repeats) {
+    *taken = *repeats = false;
     const uint64_t nb = (uint64_t)std::min(R.n, S.n);
     if (nb == 0 || nb > DJ_MAX || !direct_allowed(c) || R.host || S.host) return JN_OK;
-    if (mode == MODE_EMIT) return direct_mode<K, MODE_EMIT>(c, R, S, plan, res, taken);
-    if (mode == MODE_AGG) return direct_mode<K, MODE_AGG>(c, R, S, plan, res, taken);
-    return direct_mode<K, MODE_COUNT>(c, R, S, plan, res, taken);
+    if (mode == MODE_EMIT) return direct_mode<K, MODE_EMIT>(c, R, S, plan, res, taken, repeats);
+    if (mode == MODE_AGG) return direct_mode<K, MODE_AGG>(c, R, S, plan, res, taken, repeats);
+    return direct_mode<K, MODE_COUNT>(c, R, S, plan, res, taken, repeats);
 }
 
 template jn_status run_direct<int32_t>(jn_ctx*, const Cols<int32_t>&, const Cols<int32_t>&, int, OutPlan*, RunResult*,
-                                       bool*);
+                                       bool*, bool*);
 template jn_status run_direct<int64_t>(jn_ctx*, const Cols<int64_t>&, const Cols<int64_t>&, int, OutPlan*, RunResult*,
-                                       bool*);
+                                       bool*, bool*);
 
 // ------------------------------------------------------------------ batch --
 // Equi-joins of a batch by the same method, all of them in every launch: each

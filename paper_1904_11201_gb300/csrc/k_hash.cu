@@ -753,9 +753,10 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
         }
         return JN_OK;
     }
+    bool repeats = false;  // the build keys are known to have several rows
     if (!sort_merge) {
         bool taken = false;
-        const jn_status st = run_direct<K>(c, R, S, mode, plan, res, &taken);
+        const jn_status st = run_direct<K>(c, R, S, mode, plan, res, &taken, &repeats);
         if (st != JN_OK || taken) return st;
     }
     const jn_tuning& tu = c->tune;
@@ -1040,19 +1041,21 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             // (2^28 x 2^28 random int32 rows: 10.7 ms, 11.3 counted first and then
             // written)
             room = (rows + rows / 4 * 3) / segs + 4096;
-            if (nitems >= 4096 && rows >= (1u << 23)) {
-                // many pairs a row: one work item in 64 is counted first, so that a
-                // large join does not keep pairs only to find them again (2^28 x
-                // 2^28 rows, Zipf 0.5, 1.3e9 pairs: 16.7 ms, 28.8 without; the
-                // sample takes 0.03 ms)
+            if (nitems >= (repeats ? 512 : 4096) && (repeats || rows >= (1u << 23))) {
+                // many pairs a row: one work item in 64 (of few, in 16) is counted
+                // first, so that a large join does not keep pairs only to find
+                // them again (2^28 x 2^28 rows, Zipf 0.5, 1.3e9 pairs: 16.7 ms,
+                // 28.8 without; 2^22 x 2^24, two a key: 0.82, 0.91 without; the
+                // sample takes 0.03 ms, most of it the host's wait)
+                const uint32_t part = nitems >= 4096 ? 64 : 16;
                 PairSegs one{};
-                one.segs = 64;
+                one.segs = part;
                 one.w = 1;
                 JN_TRY(join_once(MODE_COUNT, nullptr, one));
                 uint64_t seen;
                 JN_TRY(read_back(c, reinterpret_cast<const uint64_t*>(&small->lines[0].total), &seen, 1));
                 JN_TRY(zero(c, &small->lines[0].total, 8));
-                if (64 * seen > segs * room) room = 0;
+                if (part * seen > segs * room) room = 0;
             }
             if (room && c->mem_limit && c->scratch_bytes + 2 * segs * room * sizeof(jn_pair) > c->mem_limit) {
                 room = 0;

@@ -225,7 +225,7 @@ jn_status star_direct(jn_ctx* c, const jn_table* R, const jn_table* S1, const jn
     const Cols<K> D2{static_cast<const K*>(S2->key), nullptr, S2->payload, S2->n};
     const DirectLayout<K, MODE> l1((uint64_t)S1->n), l2((uint64_t)S2->n);
     const size_t head = sizeof(DirectSmall);  // each table has its own counters
-    const DirectStage sg(n);
+    const DirectStage sg(n, DJ_ROOM_LEAST);
     const uint32_t segs = MODE == MODE_EMIT ? sg.segs : 1;
     uint64_t cap = MODE == MODE_EMIT ? sg.cap : 0;
     Scratch s(c), ss(c);
