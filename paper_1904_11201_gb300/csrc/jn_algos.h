@@ -83,7 +83,8 @@ template <typename K>
 jn_status batch_hash_prepare(jn_ctx* c, int n, const Cols<K>* Rs, const Cols<K>* Ss, std::unique_ptr<BatchRun>* run);
 
 // The same without partitioning (jn_direct.cuh), for the joins it takes;
-// count_only: the run is never asked to emit.
+// count_only: the run is never asked to emit.  *run stays empty where the
+// partitioned batch is the better one.
 bool batch_direct_takes(const jn_ctx* c, int64_t nr, int64_t ns);
 template <typename K>
 jn_status batch_direct_prepare(jn_ctx* c, int n, const Cols<K>* Rs, const Cols<K>* Ss, bool count_only,

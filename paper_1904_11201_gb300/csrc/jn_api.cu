@@ -291,8 +291,9 @@ static jn_status batch_parts(jn_ctx* c, int count, const jn_join* joins, jn_pair
     if (!part[0].empty()) {
         const jn_status st =
             batch_direct_prepare<K>(c, (int)part[0].size(), cr[0].data(), cs[0].data(), count_only, &run[0]);
-        if (st == JN_ERR_OOM) {
-            // a device too full for the tables and the pairs' room: all of them partitioned
+        if (st == JN_ERR_OOM || (st == JN_OK && !run[0])) {
+            // a device too full for the tables and the pairs' room, or joins
+            // that run better so: all of them partitioned
             c->err.clear();
             for (size_t j = 0; j < part[0].size(); j++) move_join(0, 1, j);
             part[0].clear();

@@ -180,8 +180,9 @@ __device__ __forceinline__ uint32_t dj_claim(const DirectTab<K, MODE>& t, K k) {
 // payloads, each a random access to a table or an array (int32 rows, ms for a
 // build of 2^22: 0.11 without repeats, 0.31 with).  Where that decides between
 // the direct and the partitioned join, the rows of one hash in 2^shift are
-// counted first, 1024 to 2048 of them, and their keys.  The build's kernels
-// read the counts themselves: no host round trip (25 us here) in between.
+// counted first, 1024 to 2048 of them, and their keys.  The sample's last block
+// gives the verdict, which the build's kernels read themselves: no host round
+// trip (25 us here) in between.
 constexpr int DUP_SLOTS = 4096;   // per table
 constexpr int DUP_ROWS = 2048;    // rows per tile
 struct DupCount {
@@ -208,9 +209,22 @@ struct DupTables {
         n++;
     }
 };
+// When joins are left to the partitioned join, all of them: base and the sum
+// over the tables of once[k], or again[k] where keys have more than `ratio`
+// rows, pass `most`.
+struct DupRule {
+    float base = 0, most = 0, ratio = 1;
+    float once[DUP_MANY], again[DUP_MANY];
+};
+// The sample in memory: this, a DupCount per table, slots; starts as zeros.
+struct DupHead {
+    unsigned int left;  // the verdict
+    unsigned int done;  // blocks
+    unsigned int pad[2];
+};
 template <typename K>
-inline size_t dup_bytes(int n) {  // counts, then slots: start as zeros
-    return ((size_t)n * (sizeof(DupCount) + DUP_SLOTS * sizeof(K)) + 255) & ~(size_t)255;
+inline size_t dup_bytes(int n) {
+    return (sizeof(DupHead) + (size_t)n * (sizeof(DupCount) + DUP_SLOTS * sizeof(K)) + 255) & ~(size_t)255;
 }
 
 // Not the tables' and partitions' hash: the keys looked at lie all over them.
@@ -223,10 +237,11 @@ __device__ __forceinline__ uint32_t dup_hash(int64_t k) {
     return dup_hash((int32_t)((uint32_t)k ^ (uint32_t)((uint64_t)k >> 32) * 0x9E3779B1u));
 }
 
-// counts[j] of table j; key 0 is left out.
+// Key 0 is left out.
 template <typename K>
 __global__ void __launch_bounds__(256)
-k_dup_sample(const __grid_constant__ DupTables<K> tabs, DupCount* __restrict__ counts) {
+k_dup_sample(const __grid_constant__ DupTables<K> tabs, const __grid_constant__ DupRule rule, DupHead* head) {
+    DupCount* const counts = reinterpret_cast<DupCount*>(head + 1);
     K* const slots = reinterpret_cast<K*>(counts + tabs.n);
     const uint32_t ntiles = tabs.tiles[tabs.n];
     int j = 0;
@@ -272,24 +287,38 @@ k_dup_sample(const __grid_constant__ DupTables<K> tabs, DupCount* __restrict__ c
             atomicAdd(&counts[j].keys, (unsigned long long)keys);
         }
     }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    unsigned int before = 0;
+    if (threadIdx.x == 0) before = atomicAdd(&head->done, 1u);
+    if (__shfl_sync(0xffffffffu, before, 0) != gridDim.x - 1) return;
+    __threadfence();
+    static_assert(DUP_MANY == 32, "a lane per table");
+    float cost = 0;
+    if (threadIdx.x < tabs.n) {
+        volatile DupCount* d = counts + threadIdx.x;
+        cost = (float)d->rows > rule.ratio * (float)d->keys ? rule.again[threadIdx.x] : rule.once[threadIdx.x];
+    }
+    cost = warp_sum(cost);
+    if (threadIdx.x == 0) head->left = rule.base + cost > rule.most;
 }
 
 template <typename K>
-jn_status dup_sample(jn_ctx* c, const DupTables<K>& tabs, DupCount* counts) {
+jn_status dup_sample(jn_ctx* c, const DupTables<K>& tabs, const DupRule& rule, DupHead* head) {
     const uint32_t tiles = std::max(tabs.tiles[tabs.n], 1u);
     return launch(c, K_DIRECT_BUILD, k_dup_sample<K>, dim3(std::min<uint32_t>(tiles, 8 * (uint32_t)c->num_sms)),
-                  dim3(256), 0, tabs, counts);
+                  dim3(256), 0, tabs, rule, head);
 }
 
-// A single join is left to the partitioned one: 1.8 rows a key and more.
-__device__ __forceinline__ bool dj_left(const DupCount* dup) { return dup && 5 * dup->rows > 9 * dup->keys; }
+__device__ __forceinline__ bool dj_left(const DupHead* dup) { return dup && dup->left; }
 
 // n 16-byte words set to zero by the block's share of a grid.
 __device__ __forceinline__ void dj_zero(uint4* p, uint64_t n) {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
         p[i] = make_uint4(0, 0, 0, 0);
 }
-static __global__ void __launch_bounds__(256) k_direct_zero(uint4* p, uint64_t n, const DupCount* __restrict__ dup) {
+static __global__ void __launch_bounds__(256) k_direct_zero(uint4* p, uint64_t n, const DupHead* __restrict__ dup) {
     if (!dj_left(dup)) dj_zero(p, n);
 }
 
@@ -341,7 +370,7 @@ __device__ __forceinline__ void dj_insert_rows(const K* __restrict__ key, const 
 template <typename K, int MODE>
 __global__ void __launch_bounds__(DJ_T)
 k_direct_insert(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int use_g,
-                uint2* __restrict__ where, DirectSmall* __restrict__ small, const DupCount* __restrict__ dup) {
+                uint2* __restrict__ where, DirectSmall* __restrict__ small, const DupHead* __restrict__ dup) {
     if (dj_left(dup)) return;
     dj_insert_rows<K, MODE>(key, pay, (int64_t)blockIdx.x * DJ_T, n, (int64_t)gridDim.x * DJ_T, t, use_g, where,
                             small->lines);
@@ -662,7 +691,7 @@ template <typename K, int MODE>
 __global__ void __launch_bounds__(DJ_T, JN_DJ_MINB)
 k_direct_probe(const K* __restrict__ key, const int32_t* __restrict__ pay, int64_t n, DirectTab<K, MODE> t, int swap,
                DirectSmall* __restrict__ small, jn_pair* __restrict__ out, uint32_t segs, unsigned long long cap,
-               LongRun* __restrict__ longs, const DupCount* __restrict__ dup) {
+               LongRun* __restrict__ longs, const DupHead* __restrict__ dup) {
     constexpr int TILE = DJ_T * DJ_U;
     using Out = WarpOut<2>;
     __shared__ int2 s_buf[MODE == MODE_EMIT ? DJ_T / 32 : 1][MODE == MODE_EMIT ? Out::ROOM : 1];
@@ -775,7 +804,7 @@ struct DirectLayout {
 // Launches of one table's build in `mem` (already zeroed up to lay.zeroed()).
 template <typename K, int MODE>
 jn_status direct_build(jn_ctx* c, const Cols<K>& B, int use_g, const DirectLayout<K, MODE>& lay, unsigned char* mem,
-                       DirectSmall* small, DirectTab<K, MODE>* t, const DupCount* dup = nullptr) {
+                       DirectSmall* small, DirectTab<K, MODE>* t, const DupHead* dup = nullptr) {
     t->slots = reinterpret_cast<typename DirectTab<K, MODE>::Slot*>(mem);
     t->nb = dj_buckets<K, MODE>((uint64_t)B.n);
     t->counts = reinterpret_cast<uint32_t*>(mem + lay.slots);
@@ -807,6 +836,7 @@ struct DirectStage {
         segs = np >= (1u << 23) ? DJ_SEGS : 1;
         cap = np * quarters / 4 / segs + 1024;
     }
+    uint64_t room() const { return segs * cap; }
 };
 
 // What a probe left in the counters.

@@ -59,14 +59,18 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
     JN_TRY(zero(c, mem, head + db + (look ? 0 : lay.zeroed())));
     DirectTab<K, MODE> t;
     JN_TRY(wait_copies(c, true));
-    DupCount* dup = nullptr;
+    DupHead* dup = nullptr;
     if (look) {
-        dup = reinterpret_cast<DupCount*>(mem + head);
+        dup = reinterpret_cast<DupHead*>(mem + head);
         DupTables<K> tabs{};
         tabs.add(B.key, B.n);
-        JN_TRY(dup_sample<K>(c, tabs, dup));
+        DupRule rule;
+        rule.ratio = 1.8f;
+        rule.once[0] = 0;
+        rule.again[0] = 1;
+        JN_TRY(dup_sample<K>(c, tabs, rule, dup));
         JN_TRY(launch(c, K_MEMSET, k_direct_zero, dim3(8 * (unsigned)c->num_sms), dim3(256), 0,
-                      reinterpret_cast<uint4*>(mem + head + db), (uint64_t)(lay.zeroed() / 16), (const DupCount*)dup));
+                      reinterpret_cast<uint4*>(mem + head + db), (uint64_t)(lay.zeroed() / 16), (const DupHead*)dup));
     }
     JN_TRY((direct_build<K, MODE>(c, B, swap ? 1 : 0, lay, mem + head + db, small, &t, dup)));
     auto kp = k_direct_probe<K, MODE>;
@@ -75,7 +79,7 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
     const uint64_t tiles = ceil_div(np, DJ_T * DJ_U);
     const dim3 g((unsigned)std::min<uint64_t>(tiles, (uint64_t)std::max(per, 1) * c->num_sms));
     JN_TRY(launch(c, K_DIRECT_PROBE, kp, g, dim3(DJ_T), 0, P.key, P.pay, P.n, t, swap ? 1 : 0, small, staged, segs,
-                  (unsigned long long)cap, longs, (const DupCount*)dup));
+                  (unsigned long long)cap, longs, (const DupHead*)dup));
     DirectResult r;
     JN_TRY(direct_result(c, small, segs, cap, &r));
     if (r.left) {
@@ -123,7 +127,7 @@ static jn_status direct_mode(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, OutP
         JN_TRY(zero(c, &small->lines[0].total, 8));
         JN_TRY(zero(c, &small->lines[0].longs, 4));
         JN_TRY(launch(c, K_DIRECT_PROBE, kp, g, dim3(DJ_T), 0, P.key, P.pay, P.n, t, swap ? 1 : 0, small, plan->dev,
-                      1u, (unsigned long long)total, longs, (const DupCount*)nullptr));
+                      1u, (unsigned long long)total, longs, (const DupHead*)nullptr));
         if (longs) JN_TRY(direct_long(c, longs, &small->lines[0].longs));
         JN_CUDA(c, cudaStreamSynchronize(c->stream));  // this pass reads the caller's columns
     }
@@ -150,8 +154,13 @@ template jn_status run_direct<int64_t>(jn_ctx*, const Cols<int64_t>&, const Cols
 // Equi-joins of a batch by the same method, all of them in every launch: each
 // join has its own table, its own line of counters and its own room for its
 // pairs, and the blocks take tiles of DB_ROWS rows of all joins in turn (join
-// by join, so the tables in use at a time stay in L2).
-constexpr int DB_ROWS = 4096;
+// by join, so the tables in use at a time stay in L2: the resident blocks' 1216
+// tiles are 1.2e6 rows.  With tiles of 4096 rows they were 5e6, the rows of
+// nineteen joins of 2^18, whose tables are 180 MB, and a batch of few joins had
+// too few tiles: 48 joins of 2^18 x 2^18 1.13 ms then, 0.95 now; 16 of 30000 x
+// 30000 rows with 100 rows a key 0.56 and 0.30).
+constexpr int DB_ROWS = 1024;
+constexpr int DB_CHUNK = 4096;              // pairs copied per block and round
 constexpr uint64_t DB_ROOM = 1ull << 30;  // pairs of room for a whole batch at most (8 GB)
 
 template <typename K>
@@ -188,6 +197,8 @@ struct DirectBatch {
     int32_t* runs;
     DirectLine* lines;
     LongRun* longs;  // long runs of all joins, counted in lines[0]
+    const DupHead* dup;  // the sample's verdict, or NULL
+    __device__ __forceinline__ bool left() const { return dj_left(dup); }
     __device__ __forceinline__ DirectTab<K, MODE> table(const DirectJoin<K>& d, int j) const {
         using DS = DirectSlot<K, MODE>;
         DirectTab<K, MODE> t;
@@ -203,7 +214,14 @@ struct DirectBatch {
 
 template <typename K, int MODE>
 __global__ void __launch_bounds__(DJ_T)
-k_batch_insert(DirectBatch<K, MODE> b) {
+k_batch_zero(const __grid_constant__ DirectBatch<K, MODE> b, uint4* __restrict__ p, uint64_t n) {
+    if (!b.left()) dj_zero(p, n);
+}
+
+template <typename K, int MODE>
+__global__ void __launch_bounds__(DJ_T)
+k_batch_insert(const __grid_constant__ DirectBatch<K, MODE> b) {
+    if (b.left()) return;
     const uint64_t tiles = b.btiles[b.n];
     for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         int64_t row;
@@ -217,7 +235,8 @@ k_batch_insert(DirectBatch<K, MODE> b) {
 // step 0: the runs of keys with several rows, 1: their payloads.
 template <typename K>
 __global__ void __launch_bounds__(DJ_T)
-k_batch_runs(DirectBatch<K, MODE_EMIT> b, int step) {
+k_batch_runs(const __grid_constant__ DirectBatch<K, MODE_EMIT> b, int step) {
+    if (b.left()) return;
     const uint64_t tiles = b.btiles[b.n];
     for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         int64_t row;
@@ -236,44 +255,59 @@ k_batch_runs(DirectBatch<K, MODE_EMIT> b, int step) {
 // Second pass: the joins whose pairs passed their room, to out + off[j].
 template <typename K, int MODE>
 __global__ void __launch_bounds__(DJ_T, JN_DJ_MINB)
-k_batch_probe(DirectBatch<K, MODE> b, jn_pair* __restrict__ out, const uint64_t* __restrict__ off) {
+k_batch_probe(const __grid_constant__ DirectBatch<K, MODE> b, jn_pair* __restrict__ out, const uint64_t* __restrict__ off) {
     using Out = WarpOut<2>;
     __shared__ int2 s_buf[MODE == MODE_EMIT ? DJ_T / 32 : 1][MODE == MODE_EMIT ? Out::ROOM : 1];
+    if (b.left()) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) b.lines[0].left = 1;
+        return;
+    }
     const uint64_t tiles = b.ptiles[b.n];
+    int held = -1;  // the join whose pairs or count the warp holds
+    Out wo{MODE == MODE_EMIT ? s_buf[threadIdx.x >> 5] : nullptr, nullptr, nullptr, 0, 0, b.longs, &b.lines[0].longs};
+    unsigned long long acc = 0, csum = 0;
+    auto put = [&] {
+        if (held < 0) return;
+        if (MODE == MODE_EMIT)
+            wo.flush();
+        else
+            warp_add_to(wo.cursor, acc);
+        acc = 0;
+    };
     for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         int64_t row;
         const int j = db_tile(b.ptiles, b.n, t, &row);
         const DirectJoin<K> d = b.joins[j];
-        uint64_t at = d.stage0, cap = d.cap;
-        unsigned long long* cursor = &b.lines[j].total;
-        if (MODE == MODE_EMIT && off) {
-            at = off[j];
-            cap = off[j + 1] - at;
-            if (cap <= d.cap) continue;  // already written
-            cursor = &b.lines[j].chk;    // the first pass's total stays
+        if (MODE == MODE_EMIT && off && off[j + 1] - off[j] <= d.cap) continue;  // already written
+        if (j != held) {
+            put();
+            held = j;
+            if (MODE == MODE_EMIT && off) {
+                wo.out = reinterpret_cast<int2*>(out + off[j]);
+                wo.cap = off[j + 1] - off[j];
+                wo.cursor = &b.lines[j].chk;  // the first pass's total stays
+            } else {
+                wo.out = reinterpret_cast<int2*>(out + d.stage0);
+                wo.cap = d.cap;
+                wo.cursor = &b.lines[j].total;
+            }
         }
-        Out wo{MODE == MODE_EMIT ? s_buf[threadIdx.x >> 5] : nullptr, cursor, reinterpret_cast<int2*>(out + at), cap, 0,
-               b.longs, &b.lines[0].longs};
-        unsigned long long acc = 0, csum = 0;
         dj_probe_rows<K, MODE>(d.pkey, d.ppay, row, min(d.pn, row + DB_ROWS), DJ_T * DJ_U, b.table(d, j), d.swap, wo,
                                acc, csum);
-        if (MODE == MODE_EMIT)
-            wo.flush();
-        else
-            warp_add_to(cursor, acc);
     }
+    put();
 }
 
 // The pairs of the joins that fit their room, to their place in the output:
-// DB_ROWS pairs of one join per block and round.
+// DB_CHUNK pairs of one join per block and round.
 __global__ void __launch_bounds__(256)
 k_batch_gather(const uint64_t* __restrict__ staged, const uint64_t* __restrict__ stage0,
                const uint64_t* __restrict__ off, const uint64_t* __restrict__ chunks, int n, uint64_t* __restrict__ out) {
     const uint64_t total = chunks[n];
     for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
         const int j = find_segment(chunks, n, c);
-        const uint64_t q0 = (c - chunks[j]) * DB_ROWS;
-        const uint64_t m = min((uint64_t)DB_ROWS, off[j + 1] - off[j] - q0);
+        const uint64_t q0 = (c - chunks[j]) * DB_CHUNK;
+        const uint64_t m = min((uint64_t)DB_CHUNK, off[j + 1] - off[j] - q0);
         const uint64_t* src = staged + stage0[j] + q0;
         uint64_t* dst = out + off[j] + q0;
         for (uint64_t e = threadIdx.x; e < m; e += 256) dst[e] = __ldcs(src + e);
@@ -286,9 +320,12 @@ struct DirectBatchRun : BatchRun {
     int n = 0;
     DirectBatch<K, MODE> b{};
     std::vector<DirectJoin<K>> joins;
+    std::vector<uint64_t> bt, pt;  // tile offsets; like joins, kept for the copies to the device
     jn_pair* staged = nullptr;
     uint64_t btiles = 0, ptiles = 0;
     bool fits = true;
+    bool left = false;   // the rule's verdict: nothing was done
+    uint32_t longs = 0;  // parts of long runs among the kept pairs
     std::vector<uint64_t> words;  // emit: stage0, chunk offsets
 
     dim3 grid(jn_ctx* c, const void* fn, uint64_t tiles) const {
@@ -300,12 +337,78 @@ struct DirectBatchRun : BatchRun {
         return dim3((unsigned)std::min<uint64_t>(std::max<uint64_t>(tiles, 1), (uint64_t)std::max(per, 1) * c->num_sms));
     }
 
+    // Whether the batch's equi-joins go to the partitioned batch after all, all of
+    // them: the sum of what they take here beyond what they take there, with the
+    // largest build sides' repeated keys from a sample, against what a second set
+    // of launches and the sets' own small terms take.  False: not to be asked.
+    // us per 2^20 rows on GB300, build + probe rows, from batches of joins of 2^14
+    // to 2^20 build rows: int32 keys 62 + 13 here, 90 + 28 with repeated keys,
+    // 29 a row partitioned; int64 keys 58 + 14, 75 + 33 and 46.  Joins of up to
+    // 8192 rows are not looked at: launches and latency bound both.
+    bool ask(const Cols<K>* Rs, const Cols<K>* Ss, DupTables<K>* tabs, DupRule* r) {
+        constexpr bool W = sizeof(K) == 8;
+        constexpr int64_t SMALL = 8192, LOOK = 1 << 16;  // a part of a table shows repeats too
+        std::vector<int> large;
+        double worst = 0, least = 0, all = 0, seen = 0;
+        auto rows = [&](int i, double* bn, double* pn) {
+            *bn = (double)std::min(Rs[i].n, Ss[i].n) / (1 << 20);
+            *pn = (double)std::max(Rs[i].n, Ss[i].n) / (1 << 20);
+        };
+        auto loss = [&](int i, bool again) {
+            double bn, pn;
+            rows(i, &bn, &pn);
+            return again ? (W ? 75 : 90) * bn + (W ? 33 : 28) * pn - (W ? 46 : 29) * (bn + pn)
+                         : (W ? 58 : 62) * bn + (W ? 14 : 13) * pn - (W ? 46 : 29) * (bn + pn);
+        };
+        r->most = 110;
+        for (int i = 0; i < n; i++) {
+            if (std::min(Rs[i].n, Ss[i].n) > SMALL)
+                large.push_back(i);
+            else
+                r->base += (float)loss(i, false);
+        }
+        for (int i : large) {
+            worst += std::max(loss(i, true), loss(i, false));
+            least += std::min(loss(i, true), loss(i, false));
+        }
+        if (worst + r->base <= r->most) return false;
+        if (least + r->base > r->most) {  // whatever the keys are
+            left = true;
+            return false;
+        }
+        std::sort(large.begin(), large.end(),
+                  [&](int x, int y) { return std::min(Rs[x].n, Ss[x].n) > std::min(Rs[y].n, Ss[y].n); });
+        for (size_t k = 0; k < large.size(); k++) {
+            double bn, pn;
+            rows(large[k], &bn, &pn);
+            all += bn;
+            if (k >= DUP_MANY) continue;
+            seen += bn;
+            const Cols<K>& B = Ss[large[k]].n < Rs[large[k]].n ? Ss[large[k]] : Rs[large[k]];
+            tabs->add(B.key, std::min(B.n, LOOK));
+            r->once[k] = (float)loss(large[k], false);
+            r->again[k] = (float)loss(large[k], true);
+        }
+        for (int k = 0; k < tabs->n; k++) {  // the ones looked at stand for the rest
+            r->once[k] *= (float)(all / seen);
+            r->again[k] *= (float)(all / seen);
+        }
+        return true;
+    }
+
     jn_status prepare(jn_ctx* c, const Cols<K>* Rs, const Cols<K>* Ss) {
         using DS = DirectSlot<K, MODE>;
+        DupTables<K> tabs{};
+        DupRule rule;
+        const bool asked = MODE == MODE_EMIT && ask(Rs, Ss, &tabs, &rule);
+        if (left) return JN_OK;
         s.reset(new Scratch(c));
         joins.resize(n);
-        std::vector<uint64_t> bt(n + 1, 0), pt(n + 1, 0);
-        uint64_t buckets = 0, rows = 0, stage = 0;
+        bt.assign((size_t)n + 1, 0);
+        pt.assign((size_t)n + 1, 0);
+        uint64_t buckets = 0, rows = 0, stage = 0, probed = 0;
+        for (int i = 0; i < n; i++) probed += (uint64_t)std::max(Rs[i].n, Ss[i].n);
+        const uint32_t quarters = probed > DB_ROOM / DJ_ROOM * 4 ? DJ_ROOM_LEAST : DJ_ROOM;
         for (int i = 0; i < n; i++) {
             const bool swap = Ss[i].n < Rs[i].n;
             const Cols<K>&B = swap ? Ss[i] : Rs[i], &P = swap ? Rs[i] : Ss[i];
@@ -313,7 +416,7 @@ struct DirectBatchRun : BatchRun {
             DirectJoin<K>& d = joins[i];
             d = DirectJoin<K>{B.key, B.pay, P.key, P.pay, B.n, live ? P.n : 0, buckets, rows, stage, 0, 0, swap ? 1 : 0};
             if (live) d.nb = dj_buckets<K, MODE>((uint64_t)B.n);
-            if (live && MODE == MODE_EMIT) d.cap = (uint64_t)P.n + (uint64_t)P.n / 4 + 1024;
+            if (live && MODE == MODE_EMIT) d.cap = DirectStage((uint64_t)P.n, quarters).room();
             buckets += live ? d.nb + 1 : 0;
             rows += (uint64_t)B.n;
             stage += d.cap;
@@ -334,7 +437,11 @@ struct DirectBatchRun : BatchRun {
         JN_TRY(s->get(&d_joins, (size_t)n));
         JN_TRY(s->get(&d_bt, (size_t)n + 1));
         JN_TRY(s->get(&d_pt, (size_t)n + 1));
-        JN_TRY(s->get(&zeroed, lines + slots + counts));
+        // counters and sample (128 and 256 bytes' multiples), then the tables
+        const size_t db = asked ? dup_bytes<K>(tabs.n) : 0, tables = (slots + counts + 15) & ~(size_t)15;
+        JN_TRY(s->get(&zeroed, lines + db + tables));
+        DupHead* const dup = asked ? reinterpret_cast<DupHead*>(zeroed + lines) : nullptr;
+        b.dup = dup;
         if (MODE == MODE_EMIT) {
             JN_TRY(s->get(&b.where, rows));
             JN_TRY(s->get(&b.runs, rows * (DS::COUNTS_ASIDE ? 2 : 1)));
@@ -346,17 +453,22 @@ struct DirectBatchRun : BatchRun {
         b.ptiles = d_pt;
         b.n = n;
         b.lines = reinterpret_cast<DirectLine*>(zeroed);
-        b.slots = reinterpret_cast<typename DS::T*>(zeroed + lines);  // lines are 128 bytes: aligned to a bucket
-        b.counts = reinterpret_cast<uint32_t*>(zeroed + lines + slots);
+        b.slots = reinterpret_cast<typename DS::T*>(zeroed + lines + db);  // aligned to a bucket
+        b.counts = reinterpret_cast<uint32_t*>(zeroed + lines + db + slots);
         JN_CUDA(c, cudaMemcpyAsync(d_joins, joins.data(), sizeof(DirectJoin<K>) * n, cudaMemcpyHostToDevice, c->stream));
         JN_CUDA(c, cudaMemcpyAsync(d_bt, bt.data(), 8 * (n + 1), cudaMemcpyHostToDevice, c->stream));
         JN_CUDA(c, cudaMemcpyAsync(d_pt, pt.data(), 8 * (n + 1), cudaMemcpyHostToDevice, c->stream));
-        JN_CUDA(c, cudaStreamSynchronize(c->stream));  // the host vectors go out of scope below
         GraphPhase gp(c, c->tune.graphs != 0 && !c->profiling);
         JN_TRY(gp.begin());
         jn_status st = JN_OK;
         do {
-            if ((st = zero(c, zeroed, lines + slots + counts)) != JN_OK) break;
+            if ((st = zero(c, zeroed, lines + db + (dup ? 0 : tables))) != JN_OK) break;
+            if (dup) {
+                if ((st = dup_sample<K>(c, tabs, rule, dup)) != JN_OK) break;
+                if ((st = launch(c, K_MEMSET, k_batch_zero<K, MODE>, dim3(8 * (unsigned)c->num_sms), dim3(DJ_T), 0, b,
+                                 reinterpret_cast<uint4*>(zeroed + lines + db), (uint64_t)(tables / 16))) != JN_OK)
+                    break;
+            }
             auto ki = k_batch_insert<K, MODE>;
             if ((st = launch(c, K_DIRECT_BUILD, ki, grid(c, (const void*)ki, btiles), dim3(DJ_T), 0, b)) != JN_OK) break;
             if constexpr (MODE == MODE_EMIT) {
@@ -366,23 +478,27 @@ struct DirectBatchRun : BatchRun {
                 if ((st = launch(c, K_DIRECT_BUILD, kr, g, dim3(DJ_T), 0, b, 1)) != JN_OK) break;
             }
             auto kp = k_batch_probe<K, MODE>;
-            if ((st = launch(c, K_DIRECT_PROBE, kp, grid(c, (const void*)kp, ptiles), dim3(DJ_T), 0, b, staged,
-                             (const uint64_t*)nullptr)) != JN_OK)
-                break;
-            if (b.longs) st = direct_long(c, b.longs, &b.lines[0].longs);
+            st = launch(c, K_DIRECT_PROBE, kp, grid(c, (const void*)kp, ptiles), dim3(DJ_T), 0, b, staged,
+                        (const uint64_t*)nullptr);
         } while (0);
         if (st != JN_OK) {
             gp.abort();
             return st;
         }
         JN_TRY(gp.end_and_run());
-        std::vector<uint64_t> tot(n);
-        JN_CUDA(c, cudaMemcpy2DAsync(tot.data(), 8, b.lines, sizeof(DirectLine), 8, n, cudaMemcpyDeviceToHost, c->stream));
+        constexpr int LW = DJ_LINE_WORDS;
+        std::vector<uint64_t> tot((size_t)LW * n);
+        JN_CUDA(c, cudaMemcpy2DAsync(tot.data(), 8 * LW, b.lines, sizeof(DirectLine), 8 * LW, n, cudaMemcpyDeviceToHost,
+                                     c->stream));
         JN_CUDA(c, cudaStreamSynchronize(c->stream));
+        longs = (uint32_t)(tot[4] >> 32);
+        left = (tot[5] & 0xffffffffu) != 0;
+        if (left) return JN_OK;
+        b.dup = nullptr;  // a second pass does not ask again
         offsets.assign((size_t)n + 1, 0);
         for (int i = 0; i < n; i++) {
-            offsets[i + 1] = offsets[i] + tot[i];
-            fits &= tot[i] <= joins[i].cap;
+            offsets[i + 1] = offsets[i] + tot[(size_t)LW * i];
+            fits &= tot[(size_t)LW * i] <= joins[i].cap;
         }
         total = offsets[n];
         return JN_OK;
@@ -397,13 +513,14 @@ struct DirectBatchRun : BatchRun {
             for (int i = 0; i < n; i++) {
                 const uint64_t m = offsets[i + 1] - offsets[i];
                 words[i] = joins[i].stage0;
-                chunks[i + 1] = chunks[i] + (m <= joins[i].cap ? ceil_div(m, DB_ROWS) : 0);
+                chunks[i + 1] = chunks[i] + (m <= joins[i].cap ? ceil_div(m, DB_CHUNK) : 0);
             }
             uint64_t *d_words, *d_off;
             JN_TRY(s->get(&d_words, words.size()));
             JN_TRY(s->get(&d_off, offsets.size()));
             JN_CUDA(c, cudaMemcpyAsync(d_words, words.data(), 8 * words.size(), cudaMemcpyHostToDevice, c->stream));
             JN_CUDA(c, cudaMemcpyAsync(d_off, offsets.data(), 8 * offsets.size(), cudaMemcpyHostToDevice, c->stream));
+            if (b.longs && longs) JN_TRY(direct_long(c, b.longs, &b.lines[0].longs));
             JN_TRY(launch(c, K_DIRECT_PROBE, k_batch_gather,
                           dim3((unsigned)std::min<uint64_t>(std::max<uint64_t>(chunks[n], 1), 8 * (uint64_t)c->num_sms)),
                           dim3(256), 0, reinterpret_cast<const uint64_t*>(staged), (const uint64_t*)d_words,
@@ -434,7 +551,7 @@ jn_status batch_direct_prepare(jn_ctx* c, int n, const Cols<K>* Rs, const Cols<K
         std::unique_ptr<BatchRun> own(r);
         r->n = n;
         const jn_status st = r->prepare(c, Rs, Ss);
-        if (st != JN_OK) return st;
+        if (st != JN_OK || r->left) return st;
         c->info.partitions += (uint64_t)n;
         c->info.work_items += r->ptiles;
         *run = std::move(own);
