@@ -185,6 +185,13 @@ enum NlScreen { NL_NONE = 0, NL_BAND = 1, NL_EQ_A = 2, NL_EQ_B = 3 };
 
 struct NlCounters {
     unsigned long long total, chk;
+    unsigned long long hits;  // of the sample
+};
+
+// A first pass whose sample's hits lie in [lo, hi] does nothing: the predicate
+// accepts more than it looks like, or less, and another way is faster.
+struct NlSkip {
+    unsigned long long lo = 1, hi = 0;
 };
 
 __device__ __forceinline__ uint32_t nl_hash(int32_t k) { return khash(k) >> 16; }
@@ -196,7 +203,8 @@ k_nlj_once(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* _
            const K* __restrict__ sk, const K* __restrict__ sk2, const int32_t* __restrict__ sp, int64_t ns, int op_a,
            int op_k, long long band, int tr, int screen, NlCounters* __restrict__ cnt,
            unsigned long long* __restrict__ tile_val, const uint64_t* __restrict__ tile_off, jn_pair* __restrict__ out,
-           unsigned long long cap) {
+           unsigned long long cap, NlSkip skip) {
+    if (cnt->hits >= skip.lo && cnt->hits <= skip.hi) return;
     // emit: to out[0 .. cap) through cnt->total, or, with tile_off, every tile
     // to its own place; tile_val (if given) gets the tile's pairs
     const uint64_t tile = (uint64_t)blockIdx.y * gridDim.x + blockIdx.x;
@@ -397,19 +405,28 @@ k_nlj_once(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* _
                 if (MODE != MODE_COUNT) p[j] = valid ? (sp ? sp[s] : (int32_t)s) : 0;
                 if (MODE == MODE_AGG) gs[j] = chk_g(p[j]);
             }
-            // `first` (a band alone) rules most rounds out where there is one
+            // `first` (a band alone) rules most rounds out where there is one; a
+            // warp that it ruled out four in 64 for, or fewer, stops asking (int64
+            // checksum, 2^15 x 2^18 rows, a band of 2^19 in 2^24: 9.1 ms asked
+            // throughout, 8.1)
             auto visit = [&](auto has_first, auto first, auto test) {
+                int asked = 0, ruled = 0;
+                uint32_t count = 0;  // at most four a round
                 for (int i = i0; i < rn; i++) {
                     const KPair<K> ab = s_ab[i];
-                    if (decltype(has_first)::value) {
+                    if (decltype(has_first)::value && (asked < 64 || ruled > 4)) {
                         bool any = false;
 #pragma unroll
                         for (int j = 0; j < 4; j++) any |= first(j, ab);
-                        if (!__any_sync(0xffffffffu, any)) continue;
+                        asked++;
+                        if (!__any_sync(0xffffffffu, any)) {
+                            ruled++;
+                            continue;
+                        }
                     }
                     if (MODE == MODE_COUNT) {
 #pragma unroll
-                        for (int j = 0; j < 4; j++) acc += test(j, ab);
+                        for (int j = 0; j < 4; j++) count += test(j, ab);
                         continue;
                     }
                     uint32_t mask = 0;
@@ -459,6 +476,7 @@ k_nlj_once(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* _
                         flush(NL_BUF / 2);
                     }
                 }
+                acc += count;
             };
             constexpr std::false_type all{};
             constexpr std::true_type band_first{};
@@ -496,6 +514,73 @@ k_nlj_once(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* _
     }
 }
 
+// cnt->hits += pairs that the predicate accepts among sampled rows: block x
+// compares part x of R's sample with all of S's.
+constexpr int NL_SAMPLE_R = 4096, NL_SAMPLE_S = 512, NL_SPARTS = 128;
+template <typename K, bool HAS2>
+__global__ void __launch_bounds__(NL_SAMPLE_S)
+k_nlj_sample(const K* __restrict__ rk, const K* __restrict__ rk2, int64_t nr, const K* __restrict__ sk,
+             const K* __restrict__ sk2, int64_t ns, int op_a, int op_k, long long band, NlCounters* __restrict__ cnt) {
+    constexpr int PART = NL_SAMPLE_R / NL_SPARTS;
+    __shared__ KPair<K> s_r[PART];
+    const int mr = (int)min(nr, (int64_t)NL_SAMPLE_R), ms = (int)min(ns, (int64_t)NL_SAMPLE_S);
+    const int r0 = blockIdx.x * PART, n = min(PART, mr - r0), q = threadIdx.x;
+    if (n <= 0) return;  // the whole block
+    if (q < n) {
+        const int64_t at = (int64_t)(r0 + q) * nr / mr;
+        s_r[q] = KPair<K>{rk[at], HAS2 ? rk2[at] : K(0)};
+    }
+    __syncthreads();
+    unsigned int m = 0;
+    if (q < ms) {
+        const int64_t at = (int64_t)q * ns / ms;
+        const Interval<K> ia = op_interval<K>(op_a, sk[at]);
+        Interval<K> ib{};
+        if (HAS2) ib = band >= 0 ? band_interval<K>(sk2[at], band) : op_interval<K>(op_k, sk2[at]);
+        for (int i = 0; i < n; i++) m += iv_test(ia, s_r[i].a) && (!HAS2 || iv_test(ib, s_r[i].b));
+    }
+    m = warp_sum(m);
+    if ((q & 31) == 0 && m) atomicAdd(&cnt->hits, (unsigned long long)m);
+}
+
+// An emitting run counted and then written by k_nlj, every tile to its place.
+template <typename K>
+static jn_status nlj_thin(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, const jn_pred& pr, bool has2, int tr,
+                          OutPlan* plan, RunResult* res) {
+    const dim3 grid((unsigned)ceil_div(S.n, NLJ_STILE), (unsigned)ceil_div(R.n, tr));
+    const uint64_t tiles = (uint64_t)grid.x * grid.y;
+    const size_t smem = (size_t)tr * (sizeof(K) * (has2 ? 2 : 1) + 4);
+    Scratch s(c);
+    unsigned long long* val;
+    uint64_t* off;
+    JN_TRY(s.get(&val, tiles));
+    JN_TRY(s.get(&off, tiles + 1));
+    auto pass = [&](int kid, auto kn, jn_pair* out) {
+        return launch(c, kid, kn, grid, dim3(NLJ_T), smem, R.key, R.key2, R.pay, R.n, S.key, S.key2, S.pay, S.n,
+                      pr.op_a, pr.op_k, (long long)pr.band, tr, val, (unsigned long long*)nullptr, (const uint64_t*)off,
+                      out);
+    };
+    JN_TRY(has2 ? pass(K_NLJ_COUNT, k_nlj<K, true, MODE_COUNT>, (jn_pair*)nullptr)
+                : pass(K_NLJ_COUNT, k_nlj<K, false, MODE_COUNT>, (jn_pair*)nullptr));
+    JN_TRY(scan_u64(c, reinterpret_cast<const uint64_t*>(val), off, (int64_t)tiles));
+    uint64_t total;
+    JN_TRY(read_back(c, off + tiles, &total, 1));
+    jn_run_info& info = c->info;
+    res->count = info.result = total;
+    info.partitions = info.work_items = tiles;
+    info.r_survivors = (uint64_t)R.n;
+    info.s_survivors = (uint64_t)S.n;
+    info.prefilter = 0;
+    info.cartesian_bound = (uint64_t)R.n * (uint64_t)S.n;
+    JN_TRY(out_prepare(c, s, total, *plan));
+    if (total) {
+        JN_TRY(has2 ? pass(K_NLJ_EMIT, k_nlj<K, true, MODE_EMIT>, plan->dev)
+                    : pass(K_NLJ_EMIT, k_nlj<K, false, MODE_EMIT>, plan->dev));
+        JN_CUDA(c, cudaStreamSynchronize(c->stream));  // this pass reads the caller's columns
+    }
+    return out_finish(c, total, *plan);
+}
+
 static int nlj_screen(const jn_pred& pr, bool has2) {
     return pr.op_a == JN_EQ             ? NL_EQ_A
            : has2 && pr.band >= 0       ? NL_BAND
@@ -505,14 +590,15 @@ static int nlj_screen(const jn_pred& pr, bool has2) {
 
 template <typename K, bool HAS2>
 static jn_status nlj_once(jn_ctx* c, int mode, dim3 grid, const Cols<K>& R, const Cols<K>& S, const jn_pred& pr,
-                          int tr, NlCounters* cnt, uint64_t* val, const uint64_t* off, jn_pair* out, uint64_t cap) {
+                          int tr, NlCounters* cnt, uint64_t* val, const uint64_t* off, jn_pair* out, uint64_t cap,
+                          NlSkip skip) {
     const size_t smem = (size_t)(tr + NL_R) * 4 + (size_t)tr * (2 * sizeof(K) + 4);
     auto kn = mode == MODE_EMIT  ? k_nlj_once<K, HAS2, MODE_EMIT>
               : mode == MODE_AGG ? k_nlj_once<K, HAS2, MODE_AGG>
                                  : k_nlj_once<K, HAS2, MODE_COUNT>;
     return launch(c, mode == MODE_EMIT ? K_NLJ_EMIT : K_NLJ_COUNT, kn, grid, dim3(NLJ_T), smem, R.key, R.key2, R.pay,
                   R.n, S.key, S.key2, S.pay, S.n, pr.op_a, pr.op_k, (long long)pr.band, tr, nlj_screen(pr, HAS2), cnt,
-                  reinterpret_cast<unsigned long long*>(val), off, out, (unsigned long long)cap);
+                  reinterpret_cast<unsigned long long*>(val), off, out, (unsigned long long)cap, skip);
 }
 
 template <typename K>
@@ -554,14 +640,42 @@ jn_status run_nlj(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, const jn_pred& 
         c->err.clear();
         cap = 0;
     }
-    auto pass = [&](int m, jn_pair* to, uint64_t room) {
-        return has2 ? nlj_once<K, true>(c, m, grid, R, S, pred, tr, cnt, val, off, to, room)
-                    : nlj_once<K, false>(c, m, grid, R, S, pred, tr, cnt, val, off, to, room);
+    auto pass = [&](int m, jn_pair* to, uint64_t room, NlSkip skip) {
+        return has2 ? nlj_once<K, true>(c, m, grid, R, S, pred, tr, cnt, val, off, to, room, skip)
+                    : nlj_once<K, false>(c, m, grid, R, S, pred, tr, cnt, val, off, to, room, skip);
     };
+    // Large joins are sampled (4 us), and the first pass looks at the hits: a
+    // predicate that looks selective and accepts more than the scratch holds (a
+    // wide band, few distinct keys) would be compared twice with the first
+    // time's stores on top (2^15 x 2^18 int32 rows, 3 % accepted: 12.1 ms).
+    // Counted and then written to the tiles' places, k_nlj is the faster one
+    // below one pair in eight (6.8 ms there, 8.1 here; int64 10.3 and 11.1) and
+    // k_nlj_once above (2^13 x 2^15, half accepted: 0.41 ms here, 0.57 there).
+    const double looked = (double)std::min(R.n, (int64_t)NL_SAMPLE_R) * (double)std::min(S.n, (int64_t)NL_SAMPLE_S);
+    const unsigned long long eighth = (unsigned long long)(looked / 8);
+    NlSkip skip;
+    const bool screened = nlj_screen(pred, has2) != NL_NONE;
+    if (mode == MODE_EMIT && (cap ? pairs >= (1ull << 26) : !screened && pairs >= (1ull << 30))) {
+        if (cap)
+            skip = NlSkip{(unsigned long long)((double)cap / (double)pairs * looked) + 1, ~0ull};
+        else
+            skip = NlSkip{0, eighth};
+        auto ks = has2 ? k_nlj_sample<K, true> : k_nlj_sample<K, false>;
+        JN_TRY(launch(c, K_NLJ_COUNT, ks, dim3(NL_SPARTS), dim3(NL_SAMPLE_S), 0, R.key, R.key2, R.n, S.key, S.key2, S.n,
+                      pred.op_a, pred.op_k, (long long)pred.band, cnt));
+    }
     // without scratch the first pass only counts
-    JN_TRY(pass(mode == MODE_EMIT && !cap ? (int)MODE_COUNT : mode, staged, cap));
-    uint64_t h[2];
-    JN_TRY(read_back(c, reinterpret_cast<const uint64_t*>(cnt), h, 2));
+    JN_TRY(pass(mode == MODE_EMIT && !cap ? (int)MODE_COUNT : mode, staged, cap, skip));
+    uint64_t h[3];
+    JN_TRY(read_back(c, reinterpret_cast<const uint64_t*>(cnt), h, 3));
+    if (h[2] >= skip.lo && h[2] <= skip.hi) {
+        ss.release();
+        cap = 0;
+        if (h[2] <= eighth)
+            return nlj_thin<K>(c, R, S, pred, has2, c->tune.nlj_tile_r ? c->tune.nlj_tile_r : 1024, plan, res);
+        JN_TRY(pass(MODE_COUNT, nullptr, 0, NlSkip()));
+        JN_TRY(read_back(c, reinterpret_cast<const uint64_t*>(cnt), h, 2));
+    }
     res->count = h[0];
     res->checksum = h[1];
     info.result = h[0];
@@ -589,7 +703,7 @@ jn_status run_nlj(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, const jn_pred& 
         // compared again, every tile's pairs to their place
         JN_TRY(s.get(&off, tiles + 1));
         JN_TRY(scan_u64(c, val, off, (int64_t)tiles));
-        JN_TRY(pass(MODE_EMIT, plan->dev, h[0]));
+        JN_TRY(pass(MODE_EMIT, plan->dev, h[0], NlSkip()));
         JN_CUDA(c, cudaStreamSynchronize(c->stream));  // this pass reads the caller's columns
     }
     return out_finish(c, h[0], *plan);
