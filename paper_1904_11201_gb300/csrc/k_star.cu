@@ -297,8 +297,7 @@ jn_status star_direct(jn_ctx* c, const jn_table* R, const jn_table* S1, const jn
         JN_TRY(probe(dev, 1, m));
     }
     if (copy_back) JN_CUDA(c, cudaMemcpyAsync(user, dev, m * sizeof(jn_triple), cudaMemcpyDefault, c->stream));
-    // a second pass reads the caller's columns, a host buffer is complete on return
-    if (!done || copy_back) JN_CUDA(c, cudaStreamSynchronize(c->stream));
+    JN_CUDA(c, cudaStreamSynchronize(c->stream));  // as the two joins' way: the triples are complete on return
     if (!user) *out = dev;
     *n_out = m;
     return JN_OK;
