@@ -228,6 +228,7 @@ jn_status star_direct(jn_ctx* c, const jn_table* R, const jn_table* S1, const jn
     const DirectStage sg(n, DJ_ROOM_LEAST);
     const uint32_t segs = MODE == MODE_EMIT ? sg.segs : 1;
     uint64_t cap = MODE == MODE_EMIT ? sg.cap : 0;
+    c->info = jn_run_info();
     Scratch s(c), ss(c);
     unsigned char *a = nullptr, *b = nullptr;
     jn_triple* staged = nullptr;
@@ -265,7 +266,6 @@ jn_status star_direct(jn_ctx* c, const jn_table* R, const jn_table* S1, const jn
     }
     if (MODE == MODE_EMIT && !done && m > star_most_triples(n + (uint64_t)S1->n + (uint64_t)S2->n)) return JN_OK;
     *taken = true;
-    c->info = jn_run_info();
     c->info.result = m;
     c->info.r_survivors = n;
     c->info.s_survivors = (uint64_t)S2->n;

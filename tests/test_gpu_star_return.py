@@ -33,3 +33,16 @@ def test_triples_are_complete_on_return(caller_buffer, path):
     assert stream.query()
     assert t.shape[0] == n and int(t[:, 0].to(torch.int64).sum()) == n * (n - 1) // 2
     c.close()
+
+
+def test_run_info_covers_the_scratch_held():
+    B.build()
+    c = jn.Context(0)
+    args = tables(100000, 5000)
+    jn.jn_star(c, *args)
+    info = c.run_info()
+    # two hash tables of 8-byte slots and the kept triples at least
+    assert info["hash_path"] == 3 and info["scratch_peak"] >= 2 * 5000 * 8 + 100000 * 12
+    assert jn.jn_star_count(c, *args) == info["result"]
+    assert 2 * 5000 * 8 <= c.run_info()["scratch_peak"] < info["scratch_peak"]
+    c.close()
