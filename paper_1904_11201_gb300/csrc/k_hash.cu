@@ -988,6 +988,14 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     // copied there, two segments at a time, while the next are written: page-
     // locked host buffers, n x n random int32 rows, ms (kept in scratch first):
     // 2^24 1.61 (1.73), 2^26 5.15 (5.71), 2^28 19.6 (22.0)
+    // with the full table asked for (the autotuner's choice for large uniform
+    // tables), k_part_join's shared memory holds two blocks an SM, and int32 pairs
+    // are counted and written by the batches' kernel, item by item: 2^28 x 2^28
+    // random rows tuned 10.6 ms, 11.1 by k_part_join (10.9 with its own table size)
+    const bool by_item = mode == MODE_EMIT && !sort_merge && !heavy && sizeof(K) == 4 && tu.table_rows >= cap_of<K>() &&
+                         !(plan->user_out && *plan->user_out && !is_device_pointer(*plan->user_out));
+    unsigned long long* ival = nullptr;
+    uint64_t* ioff = nullptr;
     const bool sliced = mode == MODE_EMIT && segs > 1 && rows >= (1u << 23) && plan->user_out && *plan->user_out &&
                         !is_device_pointer(*plan->user_out);
     auto join_once = [&](int m, jn_pair* to, const PairSegs& ps) -> jn_status {
@@ -1035,7 +1043,19 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             else if (b >= SJ_IDX) JN_TRY(sort(k_sort_chunks32<uint32_t>, true));
             else JN_TRY(sort(k_sort_chunks32<uint64_t>, false));
         }
-        if (mode == MODE_EMIT && !sliced && !c->admit) {
+        if (by_item) {
+            JN_TRY(s.get(&ival, nitems));
+            JN_TRY(s.get(&ioff, nitems + 1));
+            auto kc = k_hash_join<K, MODE_COUNT>;
+            const size_t smc = JoinSmem<K, MODE_COUNT>::BYTES;
+            JN_TRY(launch(c, K_HASH_COUNT, kc,
+                          dim3((unsigned)min((uint64_t)persistent_grid(c, (const void*)kc, HJ_T, smc), nitems)), dim3(HJ_T),
+                          smc, (const RW*)PR.rows, (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P),
+                          b, ival, (const uint64_t*)nullptr, (jn_pair*)nullptr, c->d_err));
+            JN_TRY(scan_u64(c, reinterpret_cast<const uint64_t*>(ival), ioff, (int64_t)nitems));
+            JN_TRY(launch(c, K_MISC, k_copy_words, dim3(1), dim3(32), 0, (const uint64_t*)(ioff + nitems),
+                          reinterpret_cast<uint64_t*>(&small->lines[0].total), 1));
+        } else if (mode == MODE_EMIT && !sliced && !c->admit) {
             // random keys on both sides match a surviving row 1.6 times; under a
             // limit that counts scratch only with place for as many bytes of output
             // (2^28 x 2^28 random int32 rows: 10.7 ms, 11.3 counted first and then
@@ -1069,7 +1089,7 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
             ps.at[i] = i * room;
             ps.cap[i] = room;
         }
-        JN_TRY(join_once(room ? MODE_EMIT : cm, staged, ps));
+        if (!by_item) JN_TRY(join_once(room ? MODE_EMIT : cm, staged, ps));
     }
     // ---- heavy keys: c_R(h) * c_S(h) pairs each ----
     uint64_t *hp = nullptr, *hpoff = nullptr, *hch = nullptr, *hchp = nullptr;
@@ -1139,7 +1159,14 @@ jn_status run_hash(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, int mode, OutP
     }));
     uint64_t copied = 0;  // pairs that are on their way to the caller's buffer
     if (normal > 0) {
-        if (room && found.fits) {
+        if (by_item) {
+            auto ke = k_hash_join<K, MODE_EMIT>;
+            const size_t sme = JoinSmem<K, MODE_EMIT>::BYTES;
+            JN_TRY(launch(c, K_HASH_EMIT, ke,
+                          dim3((unsigned)min((uint64_t)persistent_grid(c, (const void*)ke, HJ_T, sme), nitems)), dim3(HJ_T),
+                          sme, (const RW*)PR.rows, (const RW*)PS.rows, (const Item*)idesc, (const uint64_t*)(iprefix + P),
+                          b, (unsigned long long*)nullptr, (const uint64_t*)ioff, plan->dev, c->d_err));
+        } else if (room && found.fits) {
             JN_TRY((direct_gather<uint64_t, 1>(c, sort_merge ? K_SORT_EMIT : K_HASH_EMIT, staged, segs, room, found,
                                                plan->dev)));
         } else {
