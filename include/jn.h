@@ -126,7 +126,8 @@ typedef struct {
                               filter_bits, heavy, table_rows) left automatic, a hash
                               join whose smaller table has at most 2^22 rows is not
                               partitioned at all: one hash table of that table in
-                              global memory, probed by the other                        */
+                              global memory, probed by the other (pairs of int32 keys
+                              with many rows each: at most 2^21 rows)                   */
     int32_t table_rows;    /* R rows per shared-memory table of the hash and sort-merge
                               joins (the "bucket" a work item holds): 0 = the key type's
                               full table (4096 rows for int32 keys, 2048 for int64),
@@ -301,11 +302,12 @@ typedef struct {
  * are: they are out[first[i] .. first[i] + pairs[i]).  The equi-joins of a
  * batch share every phase, and so do its band joins: those with a smaller
  * side of at most 2^22 rows (and, bands, few candidates a row) one build and
- * one probe of all their tables or indexes; the others one radix or range
- * pass, one count pass and one emit pass over a single work queue of (join,
- * partition or group) items.  Every join is counted before the single exact
- * output allocation; with tuning.graphs on, each phase of the latter is
- * replayed as a CUDA graph.  This is the batched form of the
+ * one probe of all their tables or indexes; the others, and equi-joins that
+ * run better so, one radix or range pass, one count pass and one emit pass
+ * over a single work queue of (join, partition or group) items.  Every join
+ * is counted before the single exact output allocation; with tuning.graphs
+ * on, the phases up to the counts, and the latter's emit pass, are replayed
+ * as CUDA graphs.  This is the batched form of the
  * Reducer = grid hierarchy of Sec. 3.3.4: many small joins fill the GPU
  * together instead of one launch sequence each. */
 jn_status jn_batch(jn_ctx* ctx, int32_t count, const jn_join* joins, jn_pair** out, uint64_t capacity,
@@ -361,7 +363,10 @@ jn_status jn_batch_count(jn_ctx* ctx, int32_t count, const jn_join* joins, uint6
  * fastest to the context and caches it per (algorithm, key type, size class);
  * *best (may be NULL) receives it.  The knobs tried never change a result: the hash and sort-merge joins'
  * partition bits and pre-filter, the theta join's group count, the nested
- * loop's R tile.  It stands in for the hand sweep of the partition parameter
+ * loop's R tile.  The candidates are partitionings: a context tuned for tables
+ * of at most 2^22 rows, for narrow bands or for batches no longer takes the
+ * joins without partitioning that an untuned one takes there, which are often
+ * the faster ones.  It stands in for the hand sweep of the partition parameter
  * alpha in Sec. 5.1.4 and 5.2.4. */
 jn_status jn_autotune(jn_ctx* ctx, int32_t algo, const jn_table* R, const jn_table* S, const jn_pred* pred,
                       jn_tuning* best);

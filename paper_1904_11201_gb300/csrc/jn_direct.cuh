@@ -3,9 +3,9 @@
 //
 // The partition passes of the other paths exist so that a build table fits
 // shared memory.  A build table that stays in the GPU's 129 MB L2 needs none:
-// a probe row costs one 16-byte slot read from L2 (two slots to a 32-byte
-// sector) and is read from HBM once, in order, where the partitioned join
-// moves it twice and reads it four times.  The paper's hash join (Sec. 3.3.2)
+// a probe row costs one 32-byte bucket read from L2 (two or four slots) and is
+// read from HBM once, in order, where the partitioned join moves it twice and
+// reads it four times.  The paper's hash join (Sec. 3.3.2)
 // builds on "the smaller table" too (Sec. 2.3); pairs keep the (R, S) order
 // whichever side was built.
 //
@@ -41,9 +41,6 @@ namespace jnx {
 #ifndef JN_DJ_T
 #define JN_DJ_T 256
 #endif
-#ifndef JN_DJ_U
-#define JN_DJ_U 1
-#endif
 #ifndef JN_DJ_MINB
 #define JN_DJ_MINB 8
 #endif
@@ -52,7 +49,7 @@ namespace jnx {
 #endif
 constexpr int DJ_BUF = JN_DJ_BUF;  // results a probing warp collects before it writes them
 constexpr int DJ_T = JN_DJ_T;  // threads per block
-constexpr int DJ_U = JN_DJ_U;  // probe rows a thread looks up at once
+constexpr int DJ_U = 1;        // probe rows a thread looks up at once (4 and 8 measured slower)
 
 // Counters at the head of a direct join's scratch (zeroed with its table).
 // Segment r of the staged results has its cursor in lines[r].total, each in a
@@ -765,7 +762,8 @@ k_direct_gather(const T* __restrict__ staged, uint32_t segs, uint64_t cap, Direc
 // 8-byte slots, 128 MB of 16-byte ones).  Measured on GB300 against the
 // better of the partition paths, half of the probe rows matching, ms for
 // build x probe rows: int32, pairs written: 2^20 x 2^26 0.78 / 1.34, 2^22 x
-// 2^22 0.30 / 0.49, 2^22 x 2^26 0.89 / 1.37, but 2^23 x 2^25 1.19 / 1.05;
+// 2^22 0.30 / 0.49, 2^22 x 2^26 0.89 / 1.37, but 2^23 x 2^25 1.19 / 1.05 (the
+// keys without repeats; with them see DupRule);
 // counted: 2^22 x 2^26 0.51 / 1.19; int64, pairs: 2^22 x 2^22 0.34 / 0.66,
 // 2^22 x 2^26 1.23 / 2.60; checksum: 2^22 x 2^24 0.71 / 0.98, but 2^23 x
 // 2^25 1.71 / 1.64.  2^16 x 2^18: 0.07 / 0.19.

@@ -18,8 +18,11 @@
 //
 // The pass is held by shared-memory latency (dependent compare-and-swaps and
 // lookups), so a block is kept small enough, in shared memory and registers,
-// for three (emit) or four (count, aggregate) on an SM: they cover each
-// other's staging and barriers.  One S row at a time per thread beats two to
+// for three (emit) or four (count, aggregate) on an SM where its table is
+// fitted to the partitions (run_hash); they cover each other's staging and
+// barriers.  A full table of 4096 int32 rows leaves two blocks (107 KB; checksum
+// one, 123 KB), one of 2048 int64 rows two: with the full table asked for, int32
+// pairs go to k_hash_join.  One S row at a time per thread beats two to
 // four with fewer blocks.  Measured on GB300, 2^28 x 2^28 uniform int32 rows:
 // count 1.42 ms (1.65 with the kernel it replaced), checksum 2.49 (4.22), pairs
 // 4.82 with the copy (1.65 + 3.24); 2^26 x 2^26, unique R keys, half matching:
@@ -33,14 +36,8 @@
 
 namespace jnx {
 
-#ifndef JN_PJ_PU
-#define JN_PJ_PU 1
-#endif
 #ifndef JN_PJ_MINB
 #define JN_PJ_MINB 4
-#endif
-#ifndef JN_PJ_PUE
-#define JN_PJ_PUE 1
 #endif
 #ifndef JN_PJ_ENT
 #define JN_PJ_ENT 5  // entries per two rows of a full table
@@ -92,7 +89,7 @@ k_part_join(const Row<K, false>* __restrict__ rrows, const Row<K, false>* __rest
     __shared__ uint32_t tmp32[33];
     __shared__ __align__(8) uint64_t bar;
     constexpr int PER = 8;  // R rows per thread: a chunk is at most 8 * PJ_T rows
-    constexpr int PU = MODE == MODE_EMIT ? JN_PJ_PUE : JN_PJ_PU;  // S rows a thread loads at once
+    constexpr int PU = 1;   // S rows a thread loads at once (two to four measured slower)
     const int tid = threadIdx.x, lane = tid & 31;
     const uint64_t nitems = *nitems_p;
     const uint32_t seg = ps.seg();

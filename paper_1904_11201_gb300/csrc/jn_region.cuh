@@ -36,10 +36,7 @@
 
 namespace jnx {
 
-#ifndef JN_RG_T
-#define JN_RG_T 512
-#endif
-constexpr int RG_T = JN_RG_T;               // threads of the region kernels (16 rows each per int32 tile)
+constexpr int RG_T = 512;               // threads of the region kernels (16 rows each per int32 tile)
 constexpr int RG_STAGE = 65536 + 64;    // bytes per staging buffer (a tile and its 16-byte widening)
 constexpr int RG_NDMAX = 1026;          // level-1 digits at most (1024 + the heavy digit, even)
 constexpr int RG_F2MAX = 256;           // level-2 digits at most

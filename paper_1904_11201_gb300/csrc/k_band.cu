@@ -15,8 +15,9 @@
 // Every candidate is a read from L2, against one from shared memory there, so
 // windows with many candidates belong to the partitioned join.  A sample of
 // both tables estimates the candidates of a row first; past the line (below)
-// nothing is built.  Should the sample be wrong by far, the probe, which counts
-// its candidates, stops, and the join is left to the partitioned one.
+// nothing is built.  Where the buckets bring far more rows than the band, the
+// check beside the buckets' bounds leaves the join to the partitioned one; should
+// both samples be wrong by far, the probe, which counts its candidates, stops.
 //
 // Measured on GB300, 2^20 x 2^24 int32 rows, ms with (without) the index, at
 // 1, 6, 12, 24 candidates a row: count 0.38 (0.61), 0.53 (0.65), 0.70 (0.71),

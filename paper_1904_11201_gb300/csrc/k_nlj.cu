@@ -9,8 +9,9 @@
 // R value ("R.x op s" <=> R.x in [lo, hi], possibly negated), which makes the
 // inner loop a subtract and an unsigned compare per column.  The exact count
 // replaces the NB_S * NB_T per-thread buffers: jn_nested_loop compares once
-// and keeps the pairs it finds in scratch (k_nlj_once); the allocation-free
-// entry point counts per tile, scans, and compares again to write (k_nlj).
+// and keeps the pairs it finds in scratch (k_nlj_once) where that pays; the
+// allocation-free entry point counts per tile, scans, and compares again to
+// write (k_nlj).
 #include <limits.h>
 
 #include <algorithm>
@@ -35,13 +36,15 @@ struct __align__(2 * sizeof(K)) KPair {
     K a, b;
 };
 
+// The tile kernel of the allocation-free call and of runs with few pairs a tile
+// (nlj_thin).  MODE_COUNT: tile_val[tile] = its pairs; MODE_EMIT: writes them at
+// out[tile_off[tile] ..].
 template <typename K, bool HAS2, int MODE>
 __global__ void __launch_bounds__(NLJ_T)
 k_nlj(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* __restrict__ rp, int64_t nr,
       const K* __restrict__ sk, const K* __restrict__ sk2, const int32_t* __restrict__ sp, int64_t ns,
       int op_a, int op_k, long long band, int tr, unsigned long long* __restrict__ tile_val,
-      unsigned long long* __restrict__ chk, const uint64_t* __restrict__ tile_off,
-      jn_pair* __restrict__ out) {
+      const uint64_t* __restrict__ tile_off, jn_pair* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem[];
     // R tile: (a, b) pairs with a second column, else the a column alone
     K* s_a = reinterpret_cast<K*>(smem);
@@ -96,7 +99,7 @@ k_nlj(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* __rest
     const bool plain = !__any_sync(0xffffffffu, inv);
     __syncthreads();
 
-    unsigned long long acc = 0, csum = 0;
+    unsigned long long acc = 0;
     auto visit = [&](auto test) {
         for (int i = 0; i < rn; i++) {
             K a, b = 0;
@@ -123,11 +126,7 @@ k_nlj(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* __rest
                 }
             } else {
 #pragma unroll
-                for (int j = 0; j < NLJ_SPT; j++) {
-                    const bool m = test(j, a, b);
-                    acc += m;
-                    if (MODE == MODE_AGG && m) csum += chk_f(s_p[i]) * chk_g(spay[j]);
-                }
+                for (int j = 0; j < NLJ_SPT; j++) acc += test(j, a, b);
             }
         }
     };
@@ -145,10 +144,6 @@ k_nlj(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* __rest
         });
     if (MODE != MODE_EMIT) {
         const unsigned long long t = block_sum(acc, tmp64);
-        if (MODE == MODE_AGG) {
-            const unsigned long long c = block_sum(csum, tmp64);
-            if (threadIdx.x == 0 && c) atomicAdd(chk, c);
-        }
         if (threadIdx.x == 0) tile_val[tile] = t;
     }
 }
@@ -557,8 +552,7 @@ static jn_status nlj_thin(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, const j
     JN_TRY(s.get(&off, tiles + 1));
     auto pass = [&](int kid, auto kn, jn_pair* out) {
         return launch(c, kid, kn, grid, dim3(NLJ_T), smem, R.key, R.key2, R.pay, R.n, S.key, S.key2, S.pay, S.n,
-                      pr.op_a, pr.op_k, (long long)pr.band, tr, val, (unsigned long long*)nullptr, (const uint64_t*)off,
-                      out);
+                      pr.op_a, pr.op_k, (long long)pr.band, tr, val, (const uint64_t*)off, out);
     };
     JN_TRY(has2 ? pass(K_NLJ_COUNT, k_nlj<K, true, MODE_COUNT>, (jn_pair*)nullptr)
                 : pass(K_NLJ_COUNT, k_nlj<K, false, MODE_COUNT>, (jn_pair*)nullptr));
@@ -771,7 +765,6 @@ static jn_status na_run(const jn_table* R, const jn_table* S, const jn_pred& pr,
     JN_TRY(na_scratch(&base));
     unsigned long long* val = static_cast<unsigned long long*>(base);
     unsigned long long* off = val + NA_MAX_TILES;
-    unsigned long long* chk = off + NA_MAX_TILES + 1;
     const dim3 grid((unsigned)gx, (unsigned)gy);
     const size_t smem = (size_t)tr * (sizeof(K) * (HAS2 ? 2 : 1) + 4);
     const K* rk = static_cast<const K*>(R->key);
@@ -779,10 +772,9 @@ static jn_status na_run(const jn_table* R, const jn_table* S, const jn_pred& pr,
     const K* sk = static_cast<const K*>(S->key);
     const K* sk2 = static_cast<const K*>(S->key2);
     // the array keeps the previous call's contents: counts are rewritten for
-    // every tile of this call, the checksum word is cleared
-    if (cudaMemsetAsync(chk, 0, sizeof(unsigned long long), st) != cudaSuccess) return JN_ERR_CUDA;
+    // every tile of this call
     k_nlj<K, HAS2, MODE_COUNT><<<grid, NLJ_T, smem, st>>>(rk, rk2, R->payload, R->n, sk, sk2, S->payload, S->n,
-                                                          pr.op_a, pr.op_k, (long long)pr.band, tr, val, chk,
+                                                          pr.op_a, pr.op_k, (long long)pr.band, tr, val,
                                                           nullptr, nullptr);
     k_na_scan<<<1, 1024, 0, st>>>(val, (int)tiles, off);
     if (cudaGetLastError() != cudaSuccess) return JN_ERR_CUDA;
@@ -797,7 +789,7 @@ static jn_status na_run(const jn_table* R, const jn_table* S, const jn_pred& pr,
     if (total > 0) {
         k_nlj<K, HAS2, MODE_EMIT><<<grid, NLJ_T, smem, st>>>(rk, rk2, R->payload, R->n, sk, sk2, S->payload, S->n,
                                                              pr.op_a, pr.op_k, (long long)pr.band, tr, nullptr,
-                                                             nullptr, reinterpret_cast<const uint64_t*>(off), out);
+                                                             reinterpret_cast<const uint64_t*>(off), out);
         if (cudaGetLastError() != cudaSuccess) return JN_ERR_CUDA;
     }
     return JN_OK;

@@ -78,13 +78,10 @@ k_star_emit(const jn_pair* __restrict__ j1, const jn_pair* __restrict__ j2, uint
 // The counters get the triples and the pairs of the first join (the left-deep
 // plan's intermediate).  Emit: in WarpOut's manner and segments, as
 // k_direct_probe, so the 12-byte triples leave as whole lines.
-#ifndef JN_SJ_U
-#define JN_SJ_U 1
-#endif
 #ifndef JN_SJ_MINB
 #define JN_SJ_MINB 6
 #endif
-constexpr int SJ_U = JN_SJ_U;  // rows a thread looks up at once, in two tables each
+constexpr int SJ_U = 1;  // rows a thread looks up at once, in two tables each
 
 template <typename K, int MODE>
 __global__ void __launch_bounds__(DJ_T, JN_SJ_MINB)
