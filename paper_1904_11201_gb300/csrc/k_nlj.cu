@@ -400,29 +400,31 @@ k_nlj_once(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* _
                 if (MODE != MODE_COUNT) p[j] = valid ? (sp ? sp[s] : (int32_t)s) : 0;
                 if (MODE == MODE_AGG) gs[j] = chk_g(p[j]);
             }
-            // `first` (a band alone) rules most rounds out where there is one; a
-            // warp that it ruled out four in 64 for, or fewer, stops asking (int64
-            // checksum, 2^15 x 2^18 rows, a band of 2^19 in 2^24: 9.1 ms asked
-            // throughout, 8.1)
+            // `first` (a band alone) rules most rounds out where there is one.  A
+            // warp that it ruled out four in 64 for, or fewer, stops asking where
+            // that gains: counts (2^15 x 2^18 rows, a band of 2^19 in 2^24: 1.9 ms,
+            // 2.5 asked throughout; int64 3.0 and 4.5) and int32 checksums (4.7 and
+            // 5.5).  The int64 checksum's loop is the slower one without the
+            // question (10.8 and 9.1), and most pairs to write come from narrower
+            // bands.  Each kind has a loop of its own: one that carried the numbers
+            // of rounds asked and ruled out took 18.1 ms for 2^16 x 2^20 rows, a
+            // band of 24414 in 2^24, pairs kept, where 15.4 are enough, and 12.0 to
+            // count, where 9.5 are.
+            constexpr bool STOPS = MODE == MODE_COUNT || (MODE == MODE_AGG && sizeof(K) == 4);
             auto visit = [&](auto has_first, auto first, auto test) {
-                int asked = 0, ruled = 0;
                 uint32_t count = 0;  // at most four a round
-                for (int i = i0; i < rn; i++) {
+                auto round = [&](auto ask, int i) {  // whether it was ruled out
                     const KPair<K> ab = s_ab[i];
-                    if (decltype(has_first)::value && (asked < 64 || ruled > 4)) {
+                    if (decltype(ask)::value) {
                         bool any = false;
 #pragma unroll
                         for (int j = 0; j < 4; j++) any |= first(j, ab);
-                        asked++;
-                        if (!__any_sync(0xffffffffu, any)) {
-                            ruled++;
-                            continue;
-                        }
+                        if (!__any_sync(0xffffffffu, any)) return true;
                     }
                     if (MODE == MODE_COUNT) {
 #pragma unroll
                         for (int j = 0; j < 4; j++) count += test(j, ab);
-                        continue;
+                        return false;
                     }
                     uint32_t mask = 0;
 #pragma unroll
@@ -441,12 +443,12 @@ k_nlj_once(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* _
                         // pairs side by side, at the price of four ballots
                         const int32_t r = s_p[i];
                         if (__popc(__ballot_sync(0xffffffffu, __popc(mask) > 2)) <= 16) {
-                            if (!mask) continue;
+                            if (!mask) return false;
                             jn_pair* o = out + atomicAdd(&s_cur, (unsigned int)__popc(mask));
 #pragma unroll
                             for (int j = 0; j < 4; j++)
                                 if ((mask >> j) & 1u) st_pair(o++, r, p[j]);
-                            continue;
+                            return false;
                         }
                         unsigned b[4], sum = 0;
 #pragma unroll
@@ -463,14 +465,27 @@ k_nlj_once(const K* __restrict__ rk, const K* __restrict__ rk2, const int32_t* _
                             at += __popc(b[j]);
                         }
                     } else {
-                        if (!__any_sync(0xffffffffu, mask)) continue;
+                        if (!__any_sync(0xffffffffu, mask)) return false;
                         acc += __popc(mask);
 #pragma unroll
                         for (int j = 0; j < 4; j++)
                             if ((mask >> j) & 1u) put(s_p[i], p[j]);
                         flush(NL_BUF / 2);
                     }
+                    return false;
+                };
+                int i = i0;
+                if (decltype(has_first)::value && !STOPS) {
+                    for (; i < rn; i++) round(has_first, i);
+                } else if (decltype(has_first)::value) {
+                    int ruled = 0;
+#pragma unroll 1
+                    for (int end = min(rn, i0 + 64);; end = rn) {
+                        for (; i < end; i++) ruled += round(has_first, i);
+                        if (end == rn || ruled <= 4) break;
+                    }
                 }
+                for (; i < rn; i++) round(std::false_type(), i);
                 acc += count;
             };
             constexpr std::false_type all{};
