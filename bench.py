@@ -36,10 +36,11 @@ sys.path.insert(0, ROOT)
 import torch  # noqa: E402
 
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
-# Thread instructions the nested-loop kernels issue per pair evaluated with the
-# two-column band predicate (ncu smsp__thread_inst_executed.sum over 4096 x
-# 65536 pairs: 1.736e9 count pass, 1.682e9 emit pass)
-NLJ_THREAD_INSTR_PER_PAIR = {"nlj_count": 6.47, "nlj_emit": 6.27}
+# Thread instructions the nested loop's kernel issues per pair evaluated with
+# the two-column band predicate, too wide to screen (ncu
+# smsp__thread_inst_executed.sum over 2^15 x 2^18 pairs: 4.527e10 counting,
+# 6.158e10 keeping the pairs it finds)
+NLJ_THREAD_INSTR_PER_PAIR = {"nlj_count": 5.27, "nlj_emit": 7.17}
 
 
 def peaks():
@@ -531,7 +532,7 @@ def star_main(args, world, rank, local, dev, stream, jn, ctx):
                                        "dimension tables of unique keys, every fact key found"
                                        % (nf >> 20, nd >> 10),
                            "fact_rows": nf, "dimension_rows": nd, "result_triples": m,
-                           "algo": "jn_star: two hash joins (left-deep), fk2 gathered between them",
+                           "algo": "jn_star (both dimension tables probed in one pass over the fact table)",
                            "l2": "inputs larger than L2 (no flush needed)",
                            "parallelism": "replicas" if world > 1 else "1 GPU"},
                 "join_floor": {"bytes": floor, "definition": "12*|R| + 8*(|S1|+|S2|) + 12*M",
@@ -1022,10 +1023,11 @@ def main():
         del out
     info = ctx.run_info()
     if w["kind"] == "hash":
-        w["config"]["algo"] += (" (region partition: one radix pass, a block per region splits it with the "
-                                "pre-filter's bitmap slice in shared memory; count, emit)"
-                                if info.get("hash_path") == 2 else
-                                " (pre-filter bitmaps, two radix passes, count, emit)")
+        w["config"]["algo"] += {
+            1: " (pre-filter bitmaps, two radix passes, join of the partitions)",
+            2: " (region partition: one radix pass, a block per region splits it with the pre-filter's bitmap slice "
+               "in shared memory; join of the partitions)",
+            3: " (no partitions: one hash table in global memory)"}.get(info.get("hash_path"), "")
         w["config"]["table_rows"] = int(info["table_rows"])  # R rows per shared-memory table
 
     ctx.reset_stats()
@@ -1081,7 +1083,7 @@ def main():
         # compare-bound: a pass evaluates all n_R x n_S pairs.  The peak is the
         # SMs' issue rate (4 schedulers x 32 lanes per SM per clock) over the
         # thread instructions the kernel issues per pair, as ncu counted them
-        # (smsp__thread_inst_executed.sum / pairs, 4K x 64K two-column band
+        # (smsp__thread_inst_executed.sum / pairs, 32K x 256K two-column band
         # predicate of this workload, too wide to screen)
         sm_mhz = pk.get("sm_max_mhz", 2070.0)
         nsm = torch.cuda.get_device_properties(local).multi_processor_count

@@ -31,8 +31,6 @@
 
 #include <algorithm>
 
-#include <algorithm>
-
 #include "jn_algos.h"
 #include "jn_common.cuh"
 
