@@ -653,13 +653,13 @@ jn_status run_nlj(jn_ctx* c, const Cols<K>& R, const Cols<K>& S, const jn_pred& 
         return has2 ? nlj_once<K, true>(c, m, grid, R, S, pred, tr, cnt, val, off, to, room, skip)
                     : nlj_once<K, false>(c, m, grid, R, S, pred, tr, cnt, val, off, to, room, skip);
     };
-    // Large joins are sampled (4 us), and the first pass looks at the hits: a
+    // Large joins are sampled (9 us), and the first pass looks at the hits: a
     // predicate that looks selective and accepts more than the scratch holds (a
     // wide band, few distinct keys) would be compared twice with the first
     // time's stores on top (2^15 x 2^18 int32 rows, 3 % accepted: 12.1 ms).
     // Counted and then written to the tiles' places, k_nlj is the faster one
     // below one pair in eight (6.8 ms there, 8.1 here; int64 10.3 and 11.1) and
-    // k_nlj_once above (2^13 x 2^15, half accepted: 0.41 ms here, 0.57 there).
+    // k_nlj_once above (2^13 x 2^15, half accepted: 0.39 ms here, 0.57 there).
     const double looked = (double)std::min(R.n, (int64_t)NL_SAMPLE_R) * (double)std::min(S.n, (int64_t)NL_SAMPLE_S);
     const unsigned long long eighth = (unsigned long long)(looked / 8);
     NlSkip skip;
